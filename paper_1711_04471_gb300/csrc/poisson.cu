@@ -23,6 +23,12 @@ namespace gbsw {
 // Out-of-range index count of the bounds-checked debug build.
 static __device__ unsigned g_sor_bounds;
 
+}  // namespace gbsw
+
+#include "poisson_tile.cuh"
+
+namespace gbsw {
+
 unsigned long long take_bounds_poisson()
 {
     unsigned h = 0, zero = 0;
@@ -385,6 +391,144 @@ static cudaError_t launch_iterations(const PDims &d, int m, float om, float h2, 
     return err;
 }
 
+static const void *sort_kernel(int items, bool rsmem)
+{
+    switch (items) {
+    case 1: return (const void *)sor_solve_kernel<1, true>;
+    case 2: return (const void *)sor_solve_kernel<2, true>;
+    case 4: return (const void *)sor_solve_kernel<4, true>;
+    default: return rsmem ? (const void *)sor_solve_kernel<0, true> : (const void *)sor_solve_kernel<0, false>;
+    }
+}
+
+// Register tile of ty x tz rows: groups per thread (1, 2, 4) and threads, false if it is too large.
+static bool sort_small(int ty, int tz, int G, size_t cap, int *items, int *threads)
+{
+    const long long groups = (long long)ty * tz * G, halo = 2ll * (ty + tz) * G;
+    if (groups > 4 * SORT_SMALL_THREADS || halo > SORT_HALO * SORT_SMALL_THREADS ||
+        sort_smem_bytes(ty, tz, G, true, true) > cap)
+        return false;
+    *items = groups <= SORT_SMALL_THREADS ? 1 : (groups <= 2 * SORT_SMALL_THREADS ? 2 : 4);
+    const long long need = std::max((groups + *items - 1) / *items, (halo + SORT_HALO - 1) / SORT_HALO);
+    *threads = (int)std::max<size_t>(64, round_up((size_t)need, 32));
+    return true;
+}
+
+// The cut of an nx x ny x nz grid for sor_solve_kernel: of all py x pz
+// tiles that fit (one CTA per SM) the one whose half-sweep costs least, by
+// an estimate in cycles.  Register tiles: about 30 shared-memory wavefronts
+// per 32 groups, 12 per 32 halo groups, 250 for the barrier and the chain
+// of one update, 1200 for the exchange between tiles.  Other tiles: 22 per
+// 32 groups of inner rows, 60 of rim rows, 3000 for the exchange.
+static SorTilePlan sort_plan(int nx, int ny, int nz)
+{
+    SorTilePlan best{};
+    int dev = 0, coop = 0, optin = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return best;
+    }
+    const size_t cap = (size_t)std::max(0, optin);
+    const int sms = sm_count();
+    const int G = ((nx + 1) / 2 + 3) / 4;
+    double best_cost = 0.0;
+    for (int py = 1; py <= std::min(ny, sms); ++py) {
+        for (int pz = 1; pz <= std::min(nz, sms / py); ++pz) {
+            const int ty = ceil_div(ny, py), tz = ceil_div(nz, pz);
+            const bool many = py * pz > 1;
+            int items = 0, threads = 0;
+            double cost;
+            if (sort_small(ty, tz, G, cap, &items, &threads)) {
+                cost = 30.0 * ty * tz * G / 32 + 250.0 + (many ? 12.0 * 2 * (ty + tz) * G / 32 + 1200.0 : 0.0);
+            } else if (sort_smem_bytes(ty, tz, G, false, false) <= cap) {
+                const long long rim = tz > 2 ? 2 * ty + std::min(ty, 2) * (tz - 2) : (long long)ty * tz;
+                const long long inner = (long long)ty * tz - rim;
+                cost = 22.0 * inner * G / 32 + 60.0 * rim * G / 32 + (many ? 3000.0 : 400.0);
+                items = 0;
+            } else {
+                continue;
+            }
+            if (best.py && cost >= best_cost) continue;
+            best_cost = cost;
+            best.py = py;
+            best.pz = pz;
+            best.items = items;
+            best.threads = threads;
+        }
+    }
+    if (!best.py) return best;
+    const int ty = ceil_div(ny, best.py), tz = ceil_div(nz, best.pz);
+    const int nk = std::max(0, tz - 2);
+    const long long rim = nk > 0 ? 2 * ty + std::min(ty, 2) * nk : (long long)ty * tz;
+    best.G = G;
+    best.magic_g = G > 1 ? (unsigned)(((1ull << 32) + G - 1) / G) : 0u;
+    best.nseg = 1;
+    best.rim_rows = (int)rim;
+    if (best.items > 0) {
+        best.rsmem = true;
+    } else {
+        const long long units = (long long)(ty > 2 ? (ty - 1) / 2 : 0) * G;  // of one z segment
+        if (units > 0 && nk > 0) {
+            const int want = (int)std::max(1ll, std::min<long long>(nk, SORT_THREADS / units));
+            best.nseg = ceil_div(nk, ceil_div(nk, want));
+        }
+        best.threads = SORT_THREADS;
+        best.rsmem = sort_smem_bytes(ty, tz, G, true, false) <= cap;
+    }
+    best.smem = sort_smem_bytes(ty, tz, G, best.rsmem, best.items > 0);
+    const void *fn = sort_kernel(best.items, best.rsmem);
+    int per_sm = 0;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, best.threads, best.smem) != cudaSuccess ||
+        per_sm < 1) {
+        cudaGetLastError();
+        best.py = 0;
+    }
+    return best;
+}
+
+// One whole solve as a cooperative launch of sor_solve_kernel.
+gbsw_status PoissonSolver::launch_tiles(const SorTileRun &run)
+{
+    SorTileArgs A{};
+    A.d = d;
+    A.plan = plan_;
+    A.omega = (float)omega;
+    A.h2 = (float)(d.dx * d.dx);
+    A.dg = sor_diag();
+    A.b = b;
+    A.p_hi = p_hi;
+    for (int c = 0; c < 2; ++c) {
+        A.e[c] = e[c];
+        A.r[c] = r[c];
+    }
+    A.partials = partials;
+    A.rim = rim_;
+    A.rim_rows = plan_.rim_rows;
+    A.sync = sync_;
+    A.ctl = ctl;
+    const int nblocks = plan_.py * plan_.pz;
+    // register tiles: the barrier count only, the epoch goes on; others: the epoch and the tiles' counts too
+    GBSW_CUDA_TRY(cudaMemsetAsync(sync_, 0, plan_.items ? sizeof(unsigned) : (size_t)32 * (nblocks + 1) * sizeof(unsigned),
+                                  stream));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nblocks);
+    cfg.blockDim = dim3(plan_.threads);
+    cfg.dynamicSmemBytes = plan_.smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    SorTileRun r = run;
+    void *args[] = {&A, &r};
+    GBSW_CUDA_TRY(cudaLaunchKernelExC(&cfg, sort_kernel(plan_.items, plan_.rsmem), args));
+    return GBSW_OK;
+}
+
 gbsw_status PoissonSolver::init(int nx, int ny, int nz, double dx, const float *b_dev, cudaStream_t s)
 {
     d.nx = nx;
@@ -410,7 +554,19 @@ gbsw_status PoissonSolver::init(int nx, int ny, int nz, double dx, const float *
     }
     rgrid = dim3(ceil_div(nx, POI_RED_THREADS), ny, ceil_div(nz, POI_RES_PLANES));
     rblocks = (int)(rgrid.x * rgrid.y * rgrid.z);
-    GBSW_CUDA_TRY(cudaMalloc((void **)&partials, 2 * (size_t)rblocks * sizeof(double)));
+    plan_ = sort_plan(nx, ny, nz);
+    const int tiles = plan_.py * plan_.pz;
+    if (tiles > 0) {
+        const size_t words = (size_t)32 * (tiles + 1);
+        GBSW_CUDA_TRY(cudaMalloc((void **)&sync_, words * sizeof(unsigned)));
+        GBSW_CUDA_TRY(cudaMemsetAsync(sync_, 0, words * sizeof(unsigned), stream));
+        if (plan_.items) {
+            const size_t rim = (size_t)2 * tiles * 2 * plan_.rim_rows * plan_.G;
+            GBSW_CUDA_TRY(cudaMalloc((void **)&rim_, rim * sizeof(uint4)));
+            GBSW_CUDA_TRY(cudaMemsetAsync(rim_, 0, rim * sizeof(uint4), stream));
+        }
+    }
+    GBSW_CUDA_TRY(cudaMalloc((void **)&partials, 2 * (size_t)std::max(rblocks, tiles) * sizeof(double)));
     GBSW_CUDA_TRY(cudaMalloc((void **)&ctl, sizeof(PoissonCtl)));
     GBSW_CUDA_TRY(cudaMemsetAsync(ctl, 0, sizeof(PoissonCtl), stream));
     dirty_ = true;
@@ -435,6 +591,10 @@ void PoissonSolver::release()
     cudaFree(ctl);
     cudaFree(s_cache);
     cudaFree(s_ok);
+    cudaFree(rim_);
+    cudaFree(sync_);
+    rim_ = nullptr;
+    sync_ = nullptr;
     s_cache = nullptr;
     s_ok = nullptr;
     s_valid_ = false;
@@ -540,6 +700,22 @@ gbsw_status PoissonSolver::build_graph()
     return GBSW_OK;
 }
 
+int PoissonSolver::chunk() const
+{
+    int c = 1;
+    for (int x = std::min(m, SOR_CHUNK_MAX); x >= 1; --x)
+        if (m % x == 0) {
+            c = x;
+            break;
+        }
+    // An interval with no divisor near SOR_CHUNK_MAX (a prime above it, say)
+    // would give chunks of a few iterations, each paying two control
+    // kernels: take full chunks, and the check then comes at the first
+    // chunk boundary at or past the interval.
+    if (c < SOR_CHUNK_MAX / 4 && m > SOR_CHUNK_MAX) c = SOR_CHUNK_MAX;
+    return c;
+}
+
 // The solve graph with predicted checks: prelude (e = 0, first residual,
 // test), then a while node whose body is a chunk of c iterations (c the
 // largest divisor of m up to SOR_CHUNK_MAX, or SOR_CHUNK_MAX when that
@@ -555,17 +731,7 @@ gbsw_status PoissonSolver::build_graph_predicted()
     exec_ = nullptr;
     graph_ = nullptr;
 
-    int c = 1;
-    for (int x = std::min(m, SOR_CHUNK_MAX); x >= 1; --x)
-        if (m % x == 0) {
-            c = x;
-            break;
-        }
-    // An interval with no divisor near SOR_CHUNK_MAX (a prime above it, say)
-    // would give chunks of a few iterations, each paying two control
-    // kernels: take full chunks, and the check then comes at the first
-    // chunk boundary at or past the interval.
-    if (c < SOR_CHUNK_MAX / 4 && m > SOR_CHUNK_MAX) c = SOR_CHUNK_MAX;
+    const int c = chunk();
     const size_t nc = (size_t)d.cplane * (size_t)(d.nz + 2);
     const float om = (float)omega, h2 = (float)(d.dx * d.dx);
     const int nxh = (d.nx + 1) / 2;
@@ -657,6 +823,7 @@ gbsw_status PoissonSolver::build_graph_predicted()
 gbsw_status PoissonSolver::enqueue()
 {
     s_valid_ = false;  // the folds change p_hi and no stencil is stored
+    if (plan_.py) return launch_tiles(SorTileRun{0, 0, tol, max_iter, m, predict_ ? chunk() : 0, nullptr, nullptr});
     if (dirty_) {
         gbsw_status st = build_graph();
         if (st != GBSW_OK) return st;
@@ -673,6 +840,13 @@ gbsw_status PoissonSolver::enqueue_fixed(int niter, bool use_graph)
         GBSW_CUDA_TRY(cudaMalloc((void **)&s_cache, n * sizeof(double)));
         GBSW_CUDA_TRY(cudaMalloc((void **)&s_ok, sizeof(int)));
         s_valid_ = false;
+    }
+    if (plan_.py) {
+        const double *s_in = s_valid_ ? s_cache : nullptr;
+        s_valid_ = false;
+        const gbsw_status st = launch_tiles(SorTileRun{1, niter, 0.0, niter, niter, 0, s_in, s_cache});
+        s_valid_ = st == GBSW_OK;
+        return st;
     }
     // the first residual may reuse the last fixed-count solve's stencil only
     // if p_hi has not changed since

@@ -55,6 +55,22 @@ struct PoissonCtl {
     int since;        // predicted checks: iterations since the last check
 };
 
+// How a grid is cut for the solve that keeps the correction in shared
+// memory (poisson_tile.cuh, sor_solve_kernel).
+struct SorTilePlan {
+    int py, pz;          // tiles in y and z; py = 0: the grid does not fit, the sweeps run as launches
+    int G;               // 16-byte groups of a colour row
+    int nseg;            // z segments of the inner march
+    int threads;         // of a CTA
+    int rim_rows;        // rim rows of the largest tile
+    int items;           // > 0: groups per thread of a tile whose e and r live in registers
+    bool rsmem;          // r in shared memory too
+    unsigned magic_g;    // ceil(2^32 / G): t / G = umulhi(t, magic_g) for t < 2^32 / G; 0 for G = 1
+    size_t smem;         // dynamic shared memory
+};
+
+struct SorTileRun;
+
 class PoissonSolver {
 public:
     // b: device array in the padded layout (owned by the caller), read at
@@ -103,6 +119,11 @@ private:
     gbsw_status build_graph();
     gbsw_status build_graph_predicted();
     gbsw_status record_fixed(int niter, cudaStream_t s);
+    gbsw_status launch_tiles(const SorTileRun &run);
+    int chunk() const;             // iterations per chunk of the predicted checks
+    SorTilePlan plan_{};
+    uint4 *rim_ = nullptr;         // rim rows that the tiles publish
+    unsigned *sync_ = nullptr;     // grid barrier count, epoch
     cudaGraphExec_t fixed_exec_ = nullptr;
     int fixed_niter_ = -1;
     bool fixed_dirty_ = true;
