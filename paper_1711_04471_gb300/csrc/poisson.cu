@@ -212,10 +212,10 @@ poisson_resid_kernel(PDims d, const float *__restrict__ b, const double *__restr
                 s = fma(-dc, pc, nb);
                 if (s_out) s_out[pidx(d, i, j, k)] = s;
             }
-            const double bc = (double)b[pidx(d, i, j, k)];
+            const double bc = f64_from_f32(b[pidx(d, i, j, k)]);
             const double res = fma(-s, r2, bc);
             float *ra = ((i + j + k) & 1) ? r1 : r0;
-            ra[cidx(d, i, j, k)] = (float)res;
+            ra[cidx(d, i, j, k)] = f32_from_f64(res);
             rr = fma(res, res, rr);
             if (WITH_BB) bb = fma(bc, bc, bb);
         }
@@ -265,7 +265,8 @@ poisson_test_kernel(const double *__restrict__ partials, int nblocks, PoissonCtl
         ctl->rho = rho;
         const bool bad = !isfinite(rr) || !isfinite(bb) || !isfinite(rho);  // a NaN b must not look converged
         if (bad) ctl->status = DEV_NONFINITE;
-        const bool done = bad || bb < 1e-60 || rho <= tol || ctl->iters >= max_iter;
+        // (a status other than OK here: the sweeps before this check gave up a wait)
+        const bool done = ctl->status != DEV_OK || bb < 1e-60 || rho <= tol || ctl->iters >= max_iter;
         ctl->done = done ? 1 : 0;
         int next = m;
         if (predict && counting && !done && rho > 0.0 && rho < ctl->rho_prev && ctl->iters > ctl->iters_prev) {
@@ -309,7 +310,7 @@ __global__ void poisson_fold_kernel(PDims d, int colour, double *__restrict__ p_
     const int i = 2 * slot + 1 + ((colour + 1 + j + k) & 1);
     if (i > d.nx) return;
     const long long c = (long long)k * d.cplane + (long long)j * d.cpitch + SOR_SLOT0 + slot;
-    p_hi[pidx(d, i, j, k)] += (double)ec[c];
+    p_hi[pidx(d, i, j, k)] += f64_from_f32(ec[c]);
     ec[c] = 0.0f;
 }
 
@@ -402,11 +403,11 @@ static const void *sort_kernel(int items, bool rsmem)
 }
 
 // Register tile of ty x tz rows: groups per thread (1, 2, 4) and threads, false if it is too large.
-static bool sort_small(int ty, int tz, int G, size_t cap, int *items, int *threads)
+static bool sort_small(int nx, int ty, int tz, int G, size_t cap, int *items, int *threads)
 {
     const long long groups = (long long)ty * tz * G, halo = 2ll * (ty + tz) * G;
     if (groups > 4 * SORT_SMALL_THREADS || halo > SORT_HALO * SORT_SMALL_THREADS ||
-        sort_smem_bytes(ty, tz, G, true, true) > cap)
+        sort_smem_bytes(nx, ty, tz, G, true, true, false) > cap)
         return false;
     *items = groups <= SORT_SMALL_THREADS ? 1 : (groups <= 2 * SORT_SMALL_THREADS ? 2 : 4);
     const long long need = std::max((groups + *items - 1) / *items, (halo + SORT_HALO - 1) / SORT_HALO);
@@ -440,9 +441,9 @@ static SorTilePlan sort_plan(int nx, int ny, int nz)
             const bool many = py * pz > 1;
             int items = 0, threads = 0;
             double cost;
-            if (sort_small(ty, tz, G, cap, &items, &threads)) {
+            if (sort_small(nx, ty, tz, G, cap, &items, &threads)) {
                 cost = 30.0 * ty * tz * G / 32 + 250.0 + (many ? 12.0 * 2 * (ty + tz) * G / 32 + 1200.0 : 0.0);
-            } else if (sort_smem_bytes(ty, tz, G, false, false) <= cap) {
+            } else if (sort_smem_bytes(nx, ty, tz, G, false, false, false) <= cap) {
                 const long long rim = tz > 2 ? 2 * ty + std::min(ty, 2) * (tz - 2) : (long long)ty * tz;
                 const long long inner = (long long)ty * tz - rim;
                 cost = 22.0 * inner * G / 32 + 60.0 * rim * G / 32 + (many ? 3000.0 : 400.0);
@@ -463,11 +464,12 @@ static SorTilePlan sort_plan(int nx, int ny, int nz)
     const int nk = std::max(0, tz - 2);
     const long long rim = nk > 0 ? 2 * ty + std::min(ty, 2) * nk : (long long)ty * tz;
     best.G = G;
-    best.magic_g = G > 1 ? (unsigned)(((1ull << 32) + G - 1) / G) : 0u;
+    best.magic_g = sort_magic(G);
     best.nseg = 1;
     best.rim_rows = (int)rim;
     if (best.items > 0) {
         best.rsmem = true;
+        best.psm = sort_smem_bytes(nx, ty, tz, G, true, true, true) <= cap;
     } else {
         const long long units = (long long)(ty > 2 ? (ty - 1) / 2 : 0) * G;  // of one z segment
         if (units > 0 && nk > 0) {
@@ -475,9 +477,9 @@ static SorTilePlan sort_plan(int nx, int ny, int nz)
             best.nseg = ceil_div(nk, ceil_div(nk, want));
         }
         best.threads = SORT_THREADS;
-        best.rsmem = sort_smem_bytes(ty, tz, G, true, false) <= cap;
+        best.rsmem = sort_smem_bytes(nx, ty, tz, G, true, false, false) <= cap;
     }
-    best.smem = sort_smem_bytes(ty, tz, G, best.rsmem, best.items > 0);
+    best.smem = sort_smem_bytes(nx, ty, tz, G, best.rsmem, best.items > 0, best.psm);
     const void *fn = sort_kernel(best.items, best.rsmem);
     int per_sm = 0;
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) != cudaSuccess ||
@@ -489,8 +491,9 @@ static SorTilePlan sort_plan(int nx, int ny, int nz)
     return best;
 }
 
-// One whole solve as a cooperative launch of sor_solve_kernel.
-gbsw_status PoissonSolver::launch_tiles(const SorTileRun &run)
+// A cooperative launch of sor_solve_kernel: a whole solve (psm), or the
+// iterations up to the next check.
+gbsw_status PoissonSolver::launch_tiles(const SorTileRun &run, cudaStream_t stream)
 {
     SorTileArgs A{};
     A.d = d;
@@ -510,9 +513,9 @@ gbsw_status PoissonSolver::launch_tiles(const SorTileRun &run)
     A.sync = sync_;
     A.ctl = ctl;
     const int nblocks = plan_.py * plan_.pz;
-    // register tiles: the barrier count only, the epoch goes on; others: the epoch and the tiles' counts too
-    GBSW_CUDA_TRY(cudaMemsetAsync(sync_, 0, plan_.items ? sizeof(unsigned) : (size_t)32 * (nblocks + 1) * sizeof(unsigned),
-                                  stream));
+    // register tiles: the epoch goes on; others: it starts at 0 with the tiles' flags
+    const int w0 = plan_.items ? SORT_SYNC_COUNT : 0, words = plan_.items ? 1 : 32 * (nblocks + 1);
+    GBSW_CUDA_TRY(cudaMemsetAsync(sync_ + w0, 0, (size_t)words * sizeof(unsigned), stream));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nblocks);
     cfg.blockDim = dim3(plan_.threads);
@@ -624,6 +627,7 @@ void PoissonSolver::set_predicted_checks(bool on)
 
 gbsw_status PoissonSolver::build_graph()
 {
+    if (plan_.py) return build_graph_tiles();
     if (predict_) return build_graph_predicted();
     if (exec_) cudaGraphExecDestroy(exec_);
     if (graph_) cudaGraphDestroy(graph_);
@@ -695,6 +699,76 @@ gbsw_status PoissonSolver::build_graph()
     if (err != cudaSuccess) {
         record_cuda_error(err, "poisson graph build", __FILE__, __LINE__);
         return GBSW_ERR_CUDA;
+    }
+    dirty_ = false;
+    return GBSW_OK;
+}
+
+// The solve graph of a grid whose sweeps run in sor_solve_kernel but whose
+// checks are kernels of their own (several warps per FP64 lane, which the
+// solve kernel's registers do not allow): prelude (first residual, test),
+// then a while node of [iterations up to the next check and fold, residual,
+// test].
+gbsw_status PoissonSolver::build_graph_tiles()
+{
+    if (exec_) cudaGraphExecDestroy(exec_);
+    if (graph_) cudaGraphDestroy(graph_);
+    exec_ = nullptr;
+    graph_ = nullptr;
+    const int predict = predict_ ? 1 : 0;
+    cudaStream_t cs = nullptr;
+    GBSW_CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
+    cudaError_t err = cudaSuccess;
+    gbsw_status st = GBSW_OK;
+    auto chk = [&](cudaError_t e2) {
+        if (err == cudaSuccess && e2 != cudaSuccess) err = e2;
+    };
+    cudaGraphConditionalHandle handle = 0;
+    cudaGraph_t body = nullptr, out = nullptr;
+    chk(cudaGraphCreate(&graph_, 0));
+    chk(cudaGraphConditionalHandleCreate(&handle, graph_, 0, cudaGraphCondAssignDefault));
+    chk(cudaStreamBeginCaptureToGraph(cs, graph_, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+    if (err == cudaSuccess) {
+        poisson_resid_kernel<true><<<rgrid, POI_RED_THREADS, 0, cs>>>(d, b, p_hi, r[0], r[1], partials, nullptr, nullptr,
+                                                                      nullptr);
+        chk(cudaGetLastError());
+        poisson_test_kernel<true><<<1, POI_RED_THREADS, 0, cs>>>(partials, rblocks, ctl, tol, max_iter, m, 0, predict,
+                                                                  handle);
+        chk(cudaGetLastError());
+        cudaStreamCaptureStatus cst;
+        cudaGraph_t cap_graph;
+        const cudaGraphNode_t *deps = nullptr;
+        size_t ndeps = 0;
+        chk(cudaStreamGetCaptureInfo(cs, &cst, nullptr, &cap_graph, &deps, nullptr, &ndeps));
+        cudaGraphNodeParams cp = {};
+        cp.type = cudaGraphNodeTypeConditional;
+        cp.conditional.handle = handle;
+        cp.conditional.type = cudaGraphCondTypeWhile;
+        cp.conditional.size = 1;
+        cudaGraphNode_t node;
+        if (err == cudaSuccess) chk(cudaGraphAddNode(&node, cap_graph, deps, nullptr, ndeps, &cp));
+        if (err == cudaSuccess)
+            chk(cudaStreamUpdateCaptureDependencies(cs, &node, nullptr, 1, cudaStreamSetCaptureDependencies));
+        if (err == cudaSuccess) body = cp.conditional.phGraph_out[0];
+    }
+    chk(cudaStreamEndCapture(cs, &out));
+    if (err == cudaSuccess) {
+        chk(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+        if (err == cudaSuccess) {
+            st = launch_tiles(SorTileRun{0, predict ? -1 : m, 0.0, 0.0, 0, 0, predict ? chunk() : 0, nullptr, nullptr}, cs);
+            poisson_resid_kernel<false><<<rgrid, POI_RED_THREADS, 0, cs>>>(d, b, p_hi, r[0], r[1], partials, nullptr,
+                                                                           nullptr, nullptr);
+            poisson_test_kernel<true><<<1, POI_RED_THREADS, 0, cs>>>(partials, rblocks, ctl, tol, max_iter, m, 1, predict,
+                                                                      handle);
+            chk(cudaGetLastError());
+        }
+        chk(cudaStreamEndCapture(cs, &out));
+    }
+    if (err == cudaSuccess && st == GBSW_OK) chk(cudaGraphInstantiate(&exec_, graph_, 0));
+    cudaStreamDestroy(cs);
+    if (err != cudaSuccess || st != GBSW_OK) {
+        if (err != cudaSuccess) record_cuda_error(err, "poisson graph build (tiles)", __FILE__, __LINE__);
+        return st != GBSW_OK ? st : GBSW_ERR_CUDA;
     }
     dirty_ = false;
     return GBSW_OK;
@@ -823,7 +897,9 @@ gbsw_status PoissonSolver::build_graph_predicted()
 gbsw_status PoissonSolver::enqueue()
 {
     s_valid_ = false;  // the folds change p_hi and no stencil is stored
-    if (plan_.py) return launch_tiles(SorTileRun{0, 0, tol, max_iter, m, predict_ ? chunk() : 0, nullptr, nullptr});
+    if (plan_.psm)
+        return launch_tiles(SorTileRun{0, 0, tol, tol * tol * (1.0 + 1e-12), max_iter, m, predict_ ? chunk() : 0, nullptr,
+                                       nullptr}, stream);
     if (dirty_) {
         gbsw_status st = build_graph();
         if (st != GBSW_OK) return st;
@@ -841,10 +917,10 @@ gbsw_status PoissonSolver::enqueue_fixed(int niter, bool use_graph)
         GBSW_CUDA_TRY(cudaMalloc((void **)&s_ok, sizeof(int)));
         s_valid_ = false;
     }
-    if (plan_.py) {
+    if (plan_.psm) {
         const double *s_in = s_valid_ ? s_cache : nullptr;
         s_valid_ = false;
-        const gbsw_status st = launch_tiles(SorTileRun{1, niter, 0.0, niter, niter, 0, s_in, s_cache});
+        const gbsw_status st = launch_tiles(SorTileRun{1, niter, 0.0, 0.0, niter, niter, 0, s_in, s_cache}, stream);
         s_valid_ = st == GBSW_OK;
         return st;
     }
@@ -890,18 +966,25 @@ gbsw_status PoissonSolver::record_fixed(int niter, cudaStream_t stream)
     const size_t nc = (size_t)d.cplane * (size_t)(d.nz + 2);
     const float om = (float)omega, h2 = (float)(d.dx * d.dx);
     const dim3 fgrid(ceil_div((d.nx + 1) / 2, 128), d.ny, d.nz), fblock(128);
-    GBSW_CUDA_TRY(cudaMemsetAsync(e[0], 0, nc * sizeof(float), stream));
-    GBSW_CUDA_TRY(cudaMemsetAsync(e[1], 0, nc * sizeof(float), stream));
+    if (!plan_.py) {
+        GBSW_CUDA_TRY(cudaMemsetAsync(e[0], 0, nc * sizeof(float), stream));
+        GBSW_CUDA_TRY(cudaMemsetAsync(e[1], 0, nc * sizeof(float), stream));
+    }
     poisson_resid_kernel<true><<<rgrid, POI_RED_THREADS, 0, stream>>>(d, b, p_hi, r[0], r[1], partials, s_cache, s_ok,
                                                                       nullptr);
     poisson_test_kernel<false><<<1, POI_RED_THREADS, 0, stream>>>(partials, rblocks, ctl, 0.0, niter, 0, 0, 0, 0);
-    cudaError_t err = launch_iterations(d, niter, om, h2, e, r, stream);
-    if (err != cudaSuccess) {
-        record_cuda_error(err, "SOR sweep launch", __FILE__, __LINE__);
-        return GBSW_ERR_CUDA;
+    if (plan_.py) {
+        const gbsw_status st = launch_tiles(SorTileRun{0, niter, 0.0, 0.0, 0, 0, 0, nullptr, nullptr}, stream);
+        if (st != GBSW_OK) return st;
+    } else {
+        cudaError_t err = launch_iterations(d, niter, om, h2, e, r, stream);
+        if (err != cudaSuccess) {
+            record_cuda_error(err, "SOR sweep launch", __FILE__, __LINE__);
+            return GBSW_ERR_CUDA;
+        }
+        poisson_fold_kernel<<<fgrid, fblock, 0, stream>>>(d, 0, p_hi, e[0]);
+        poisson_fold_kernel<<<fgrid, fblock, 0, stream>>>(d, 1, p_hi, e[1]);
     }
-    poisson_fold_kernel<<<fgrid, fblock, 0, stream>>>(d, 0, p_hi, e[0]);
-    poisson_fold_kernel<<<fgrid, fblock, 0, stream>>>(d, 1, p_hi, e[1]);
     poisson_resid_kernel<false><<<rgrid, POI_RED_THREADS, 0, stream>>>(d, b, p_hi, r[0], r[1], partials, nullptr,
                                                                        nullptr, s_cache);
     poisson_test_kernel<false><<<1, POI_RED_THREADS, 0, stream>>>(partials, rblocks, ctl, 0.0, niter, niter,

@@ -65,6 +65,7 @@ struct SorTilePlan {
     int rim_rows;        // rim rows of the largest tile
     int items;           // > 0: groups per thread of a tile whose e and r live in registers
     bool rsmem;          // r in shared memory too
+    bool psm;            // and the FP64 pressure (register tiles)
     unsigned magic_g;    // ceil(2^32 / G): t / G = umulhi(t, magic_g) for t < 2^32 / G; 0 for G = 1
     size_t smem;         // dynamic shared memory
 };
@@ -118,8 +119,9 @@ public:
 private:
     gbsw_status build_graph();
     gbsw_status build_graph_predicted();
+    gbsw_status build_graph_tiles();
     gbsw_status record_fixed(int niter, cudaStream_t s);
-    gbsw_status launch_tiles(const SorTileRun &run);
+    gbsw_status launch_tiles(const SorTileRun &run, cudaStream_t s);
     int chunk() const;             // iterations per chunk of the predicted checks
     SorTilePlan plan_{};
     uint4 *rim_ = nullptr;         // rim rows that the tiles publish
@@ -173,6 +175,30 @@ __device__ __forceinline__ float sor_div(float x, float d, float y)
     const float q = __fmul_rn(x, y);
     const float r = __fmaf_rn(-q, d, x);
     return r == 0.0f ? q : __fmaf_rn(r, y, q);
+}
+
+// One FP64 instruction costs this GPU as much time as 64 FP32 or integer
+// ones, so the checks convert between FP32 and FP64 with integer operations.
+
+// (double)x without the FP64 pipe for normal x and 0 (exact).
+__device__ __forceinline__ double f64_from_f32(float x)
+{
+    const unsigned b = __float_as_uint(x), a = b & 0x7fffffffu;
+    if (a - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(b << 29));
+    return a == 0 ? __hiloint2double((int)b, 0) : (double)x;
+}
+
+// (float)x, rounded to nearest even, without the FP64 pipe where the result is normal or 0.
+__device__ __forceinline__ float f32_from_f64(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned a = hi & 0x7fffffffu;
+    if (a - (897u << 20) < (253u << 20)) {
+        const unsigned f = ((a - (896u << 20)) << 3) | (lo >> 29);
+        return __uint_as_float((f + (((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29)) | (hi & 0x80000000u));
+    }
+    return (a | lo) == 0 ? __uint_as_float(hi) : (float)x;
 }
 
 }  // namespace gbsw

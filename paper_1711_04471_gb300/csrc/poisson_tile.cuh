@@ -30,12 +30,20 @@
 // first and is published with one flag count per warp; a neighbour looks at
 // the flags in the middle of its march and reads the rows ahead.
 //
-// Residual checks meet at a grid barrier.  Every wait is bounded by a clock
+// Every wait is bounded by a clock
 // budget; a wait that gives up records DEV_TIMEOUT and the CTA returns.
 //
 // Measured, us per iteration (half-sweep launches before, this kernel):
-// 256x256x128 16.6, 13.5; 300x300x90 18.6, 14.5; 256x128x64 8.9, 6.1;
-// 160x96x64 9.9, 3.2; 72x48x40 5.4, 2.3; 16x16x12 4.7, 0.76 (one CTA).
+// 256x256x128 16.6, 13.1; 300x300x90 18.6, 14.0; 256x128x64 8.9, 5.1;
+// 160x96x64 9.9, 3.2; 72x48x40 5.4, 2.2; 16x16x12 4.7, 0.80 (one CTA).
+//
+// Checks.  A register tile whose FP64 pressure and right-hand side fit in
+// shared memory too (psm, about 2 M cells) runs the whole solve in one
+// launch: the FP64 residual of a 160x96x64 grid and its way through the grid
+// barriers take about 20 us, three kernels and a loop node took 50. Larger
+// grids keep the residual as a kernel of its own in a graph's loop: it is
+// bound by the FP64 pipe and wants the warps that this kernel's registers
+// do not allow (0.20 ms against 0.13 at 256x256x128).
 //
 // Arithmetic.  Every update is that of sor_sweep_kernel, operation by
 // operation, so the iterates are bitwise the same; the residual norms are
@@ -56,11 +64,17 @@ constexpr int SORT_KINDS = 16;              // kinds of group by their diagonals
 constexpr int SORT_RB = 4;                  // rim items of a thread in flight
 constexpr long long SORT_WAIT_CYCLES = 4000000000LL;
 
+// Words of SorTileArgs::sync.  The epoch (of the last half-sweep so far) goes
+// on from launch to launch of a register tile's solver; the others are 0 at launch.
+constexpr int SORT_SYNC_EPOCH = 0;
+constexpr int SORT_SYNC_COUNT = 1;    // CTAs that have come to a grid barrier
+
 // How a solve ends and where its checks come.
 struct SorTileRun {
     int fixed;        // 1: exactly n iterations (max_iter), no test
     int n;            // fixed: iterations
     double tol;
+    double tol2_above;  // a bound above tol^2: a larger ratio of the square sums is not converged
     int max_iter;
     int m;            // check interval
     int chunk;        // predicted checks: iterations are counted in chunks (0: check every m)
@@ -79,7 +93,7 @@ struct SorTileArgs {
     double *partials;     // 2 per CTA
     uint4 *rim;           // published rim rows: [colour][tile][half][rim row][group]
     int rim_rows;         // rim rows of the largest tile
-    unsigned *sync;       // word 0: grid barrier count (0 at launch), word 1: epoch of the last half-sweep so far
+    unsigned *sync;       // SORT_SYNC_* words, then from word 32 a flag per tile, 32 words apart
     PoissonCtl *ctl;
 };
 
@@ -96,11 +110,13 @@ struct SorRimRow {
 // Dynamic shared memory of a tile of ty x tz rows: e (and r) of both
 // colours, then the rim rows; of a register tile: e with its halo, r and
 // the diagonals.
-inline size_t sort_smem_bytes(int ty, int tz, int G, bool rsmem, bool regs)
+// With psm also the FP64 pressure of a register tile with its halo, and b.
+inline size_t sort_smem_bytes(int nx, int ty, int tz, int G, bool rsmem, bool regs, bool psm)
 {
     const size_t rows = (size_t)ty * tz;
     const size_t fixed = SORT_TILE_BYTES + SORT_KINDS * 32;
-    if (regs) return fixed + ((size_t)(ty + 2) * (tz + 2) + rows) * G * 32;
+    const size_t padded = (size_t)(ty + 2) * (tz + 2);
+    if (regs) return fixed + (padded + rows) * G * 32 + (psm ? (padded * 8 + rows * 4) * nx : 0);
     return fixed + rows * G * 32 * (rsmem ? 2 : 1) + (size_t)(2 * (ty + tz)) * sizeof(SorRimRow);
 }
 
@@ -110,7 +126,7 @@ inline size_t sort_smem_bytes(int ty, int tz, int G, bool rsmem, bool regs)
 struct SorTile {
     SorTileArgs A;
     int G, threads;
-    unsigned magic_g;
+    unsigned magic_g, magic_nx, magic_ty, magic_slots;  // of divisions by G, nx, ty and the slots of a row
     int ta, tb, py, ntiles;  // place of the tile
     int j0, k0, k1;          // first row, first and last plane
     int ty, tz, nrow;        // rows in y, planes, rows of the tile
@@ -170,7 +186,12 @@ __device__ __forceinline__ void st_relaxed_2x64(uint4 *p, float a, float b, unsi
                  "l"(e | __float_as_uint(b)) : "memory");
 }
 
-__device__ __forceinline__ int sort_div_g(unsigned magic, unsigned t) { return magic ? (int)__umulhi(t, magic) : (int)t; }
+// t / n for t n < 2^32 by a multiplication: magic = ceil(2^32 / n), 0 for n = 1.
+__host__ __device__ inline unsigned sort_magic(unsigned n)
+{
+    return n > 1 ? (unsigned)(((1ull << 32) + n - 1) / n) : 0u;
+}
+__device__ __forceinline__ int sort_div(unsigned magic, unsigned t) { return magic ? (int)__umulhi(t, magic) : (int)t; }
 
 // Row t of a tile's rim rows: jl | kl << 16 (the inverse of sort_rim_index).
 __device__ __forceinline__ int sort_row_of(int t, int ty, int tz)
@@ -330,12 +351,13 @@ __device__ __noinline__ bool sort_grid_barrier()
 {
     SorTile &T = sort_tile();
     __syncthreads();
+    if (gridDim.x == 1) return true;
     bool late = false;
     if (threadIdx.x == 0) {
         const unsigned n = ++T.barriers;
         fence_gpu();
-        atomicAdd(T.A.sync, 1u);
-        late = !wait_reached(T.A.sync, n * gridDim.x);
+        atomicAdd(T.A.sync + SORT_SYNC_COUNT, 1u);
+        late = !wait_reached(T.A.sync + SORT_SYNC_COUNT, n * gridDim.x);
         fence_gpu();
     }
     return !__syncthreads_or(late);
@@ -394,79 +416,105 @@ __device__ __forceinline__ float4 sort_far_get(const uint4 *from, int half, unsi
     return make_float4(__uint_as_float(f.a.x), __uint_as_float(f.a.z), __uint_as_float(f.b.x), __uint_as_float(f.b.z));
 }
 
-// r = b - A p_hi in FP64 on the tile (as poisson_resid_kernel, bitwise);
-// partial sums of r^2 and, with with_bb, of b^2.  A thread takes columns
-// (i, j) and marches in z, its reads one plane ahead.
-template <bool RSMEM>
+// Of a register tile (psm): the FP64 pressure with its halo and the right-hand side, in shared memory.
+__device__ __forceinline__ double *sort_p(const SorTile &T)
+{
+    return reinterpret_cast<double *>(sort_diags(T, true) + SORT_KINDS);
+}
+__device__ __forceinline__ float *sort_b(const SorTile &T)
+{
+    return reinterpret_cast<float *>(sort_p(T) + (T.ty + 2) * (T.tz + 2) * T.A.d.nx);
+}
+
+// r = b - A p_hi in FP64 on the tile (as poisson_resid_kernel, bitwise), and
+// the partial sums of r^2 and, with with_bb, of b^2.  s_in: the stencil is
+// read, s_out: it is stored (FP64, padded layout).  p and b are in shared
+// memory but for the halo; a thread takes single cells (dense over the tile:
+// the FP64 pipe is the bound, and half-empty warps cost it as much as full
+// ones), two at a time.
 __device__ __noinline__ void sort_residual(const double *s_in, double *s_out, bool with_bb)
 {
     SorTile &T = sort_tile();
-    const PDims d = T.A.d;
-    const int j0 = T.j0, k0 = T.k0, k1 = T.k1, ty = T.ty, G = T.G;
+    const PDims &d = T.A.d;
+    const int j0 = T.j0, k0 = T.k0, ty = T.ty, tz = T.tz, G = T.G, nx = d.nx;
     const double *p_hi = T.A.p_hi;
-    const float *b = T.A.b;
     const double r2 = d.rdx2;
     double rr = 0.0, bb = 0.0;
-    const int cols = ty * d.nx;
-    for (int t = threadIdx.x; t < cols; t += blockDim.x) {
-        const int jl = t / d.nx, i = t - jl * d.nx + 1, j = j0 + jl;
-        const long long row = (long long)j * d.pitch + i;
-        const long long dm = (long long)((j == 1 ? d.ny : j - 1) - j) * d.pitch;
-        const long long dp = (long long)((j == d.ny ? 1 : j + 1) - j) * d.pitch;
-        auto P_at = [&](long long c) -> double { return SORT_OKP(c) ? p_hi[c] : 0.0; };
-        struct Plane {
-            double pn, pw, pe, ps, pt;
-            float b;
-        };
-        auto fetch = [&](int k) {
-            Plane f;
-            const long long c = (long long)k * d.plane + row;
-            f.b = SORT_OKP(c) ? b[c] : 0.0f;
-            if (s_in) {
-                f.pn = SORT_OKP(c) ? s_in[c] : 0.0;
-                f.pw = f.pe = f.ps = f.pt = 0.0;
-            } else {
-                f.pn = k < d.nz ? P_at(c + d.plane) : 0.0;
-                f.pw = i > 1 ? P_at(c - 1) : 0.0;
-                f.pe = i < d.nx ? P_at(c + 1) : 0.0;
-                f.ps = P_at(c + dm);
-                f.pt = P_at(c + dp);
+    if (!s_in && T.ntiles > 1) {
+        // the halo: rows of the neighbouring tiles (or this one's own other side), 0 outside the grid in z
+        double *P = sort_p(T);
+        const int n = 2 * (ty + tz) * nx;
+        for (int t0 = threadIdx.x; t0 < n; t0 += 4 * blockDim.x) {
+            double v[4];
+            int at[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const int t = t0 + m * blockDim.x;
+                at[m] = -1;
+                if (t < n) {
+                    const int row = sort_div(T.magic_nx, t), i = t - row * nx;
+                    int jl, kl;
+                    if (row < 2 * tz) {
+                        jl = row < tz ? -1 : ty;
+                        kl = row < tz ? row : row - tz;
+                    } else {
+                        kl = row < 2 * tz + ty ? -1 : tz;
+                        jl = row - 2 * tz - (kl < 0 ? 0 : ty);
+                    }
+                    const int k = k0 + kl;
+                    int j = j0 + jl;
+                    j = j < 1 ? d.ny : (j > d.ny ? 1 : j);
+                    const long long c = (long long)k * d.plane + (long long)j * d.pitch + i + 1;
+                    at[m] = ((kl + 1) * (ty + 2) + jl + 1) * nx + i;
+                    v[m] = k >= 1 && k <= d.nz && SORT_OKP(c) ? __ldcg(p_hi + c) : 0.0;
+                }
             }
-            return f;
-        };
-        double pm = 0.0, pc = 0.0;
-        if (!s_in) {
-            pm = k0 > 1 ? P_at((long long)(k0 - 1) * d.plane + row) : 0.0;
-            pc = P_at((long long)k0 * d.plane + row);
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+                if (at[m] >= 0) P[at[m]] = v[m];
         }
-        Plane f = fetch(k0);
-        for (int k = k0; k <= k1; ++k) {
-            const long long c = (long long)k * d.plane + row;
-            const Plane v = f;
-            if (k < k1) f = fetch(k + 1);
-            double s;
-            if (s_in) {
-                s = v.pn;
-            } else {
-                const double nb = (v.pw + v.pe) + (v.ps + v.pt) + (pm + v.pn);
-                const int dci = 6 - (i == 1) - (k == 1) - (k == d.nz) + (i == d.nx);
-                const double dc = dci == 6 ? 6.0 : (dci == 5 ? 5.0 : (dci == 7 ? 7.0 : 4.0));
-                s = fma(-dc, pc, nb);
-                if (s_out && SORT_OKP(c)) s_out[c] = s;
-                pm = pc;
-                pc = v.pn;
+        __syncthreads();
+    }
+    const int dk = (ty + 2) * nx, n = T.nrow * nx;
+    const double *P = sort_p(T);
+    const float *B = sort_b(T);
+    float *const R0 = reinterpret_cast<float *>(sort_r(T, 0));
+    const int other = 4 * T.nrow * G;
+    for (int t0 = threadIdx.x; t0 < n; t0 += 2 * blockDim.x) {
+        double res[2], bc[2];
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            const int t = t0 + m * blockDim.x;
+            res[m] = bc[m] = 0.0;
+            if (t < n) {
+                const int row = sort_div(T.magic_nx, t), i = t - row * nx + 1, kl = sort_div(T.magic_ty, row);
+                const int jl = row - kl * ty, k = k0 + kl;
+                double s;
+                const long long c = (long long)k * d.plane + (long long)(j0 + jl) * d.pitch + i;
+                if (s_in) {
+                    s = SORT_OKP(c) ? s_in[c] : 0.0;
+                } else {
+                    const double *q = P + ((kl + 1) * (ty + 2) + jl + 1) * nx + i - 1;
+                    // one tile: the rows below the first and above the last are its own other side
+                    const int down = T.ntiles == 1 && jl == 0 ? (ty - 1) * nx : -nx;
+                    const int up = T.ntiles == 1 && jl == ty - 1 ? -(ty - 1) * nx : nx;
+                    const double w = i > 1 ? q[-1] : 0.0, e = i < nx ? q[1] : 0.0;
+                    const double nb = (w + e) + (q[down] + q[up]) + (q[-dk] + q[dk]);
+                    const int dci = 6 - (i == 1) - (k == 1) - (k == d.nz) + (i == nx);
+                    const double dc = dci == 6 ? 6.0 : (dci == 5 ? 5.0 : (dci == 7 ? 7.0 : 4.0));
+                    s = fma(-dc, q[0], nb);
+                    if (s_out && SORT_OKP(c)) s_out[c] = s;
+                }
+                bc[m] = f64_from_f32(B[t]);
+                res[m] = fma(-s, r2, bc[m]);
+                R0[(((i + j0 + jl + k) & 1) ? other : 0) + 4 * row * G + ((i - 1) >> 1)] = f32_from_f64(res[m]);
             }
-            const double bc = (double)v.b;
-            const double res = fma(-s, r2, bc);
-            const int col = (i + j + k) & 1, slot = (i - 1) >> 1;
-            if (RSMEM) {
-                reinterpret_cast<float *>(sort_r(T, col))[4 * ((k - k0) * ty + jl) * G + slot] = (float)res;
-            } else {
-                const long long rc = (long long)k * d.cplane + (long long)j * d.cpitch + SOR_SLOT0 + slot;
-                if (SORT_OK1(rc)) (col ? T.A.r[1] : T.A.r[0])[rc] = (float)res;
-            }
-            rr = fma(res, res, rr);
-            if (with_bb) bb = fma(bc, bc, bb);
+        }
+        rr = fma(res[0], res[0], rr);
+        rr = fma(res[1], res[1], rr);
+        if (with_bb) {
+            bb = fma(bc[0], bc[0], bb);
+            bb = fma(bc[1], bc[1], bb);
         }
     }
     rr = sort_block_sum(rr, T.red);
@@ -477,31 +525,124 @@ __device__ __noinline__ void sort_residual(const double *s_in, double *s_out, bo
     }
 }
 
-// p_hi += e on the tile, e = 0.
-__device__ __noinline__ void sort_fold()
+// r of the tile into shared memory (a solve whose checks are kernels of their own).
+__device__ __noinline__ void sort_read_r()
 {
     SorTile &T = sort_tile();
-    const PDims d = T.A.d;
-    const int slots = (d.nx + 1) >> 1, ty = T.ty, G = T.G, ps = T.ps, e0 = T.e0;
-    double *p_hi = T.A.p_hi;
-    const float *E0 = reinterpret_cast<const float *>(sort_e(T, 0));
-    const int other = 4 * T.ncol;
-    for (int t = threadIdx.x; t < T.nrow * slots; t += blockDim.x) {
-        const int row = t / slots, s = t - row * slots;
-        const int kl = row / ty, jl = row - kl * ty;
-        const int i = 2 * s + 1;
-        const long long c = (long long)(T.k0 + kl) * d.plane + (long long)(T.j0 + jl) * d.pitch + i;
-        // cell i is of colour (i + j + k) & 1, cell i + 1 of the other
-        const int c0 = (i + T.j0 + jl + T.k0 + kl) & 1;
-        const int at = 4 * (e0 + kl * ps + jl * G) + s;
-        const float ea = E0[at + (c0 ? other : 0)], eb = E0[at + (c0 ? 0 : other)];
-        if (SORT_OKP(c)) p_hi[c] += (double)ea;
-        if (i + 1 <= d.nx && SORT_OKP(c + 1)) p_hi[c + 1] += (double)eb;
+    const PDims &d = T.A.d;
+    const int G = T.G, n = T.nrow * G, ty = T.ty;
+    for (int t = threadIdx.x; t < 2 * n; t += blockDim.x) {
+        const int colour = t >= n, u = t - colour * n;
+        const int row = sort_div(T.magic_g, u), g = u - row * G, kl = sort_div(T.magic_ty, row), jl = row - kl * ty;
+        const long long c = (long long)(T.k0 + kl) * d.cplane + (long long)(T.j0 + jl) * d.cpitch + SOR_SLOT0 + 4 * g;
+        sort_r(T, colour)[u] = SORT_OK4(c) ? __ldcg(reinterpret_cast<const float4 *>(T.A.r[colour] + c))
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
     }
+}
+
+// With psm, before the first residual: the tile's copies of p and b.
+__device__ __noinline__ void sort_read_tile()
+{
+    SorTile &T = sort_tile();
+    const PDims &d = T.A.d;
+    const int nx = d.nx, ty = T.ty;
+    double *P = sort_p(T);
+    float *B = sort_b(T);
+    for (int t = threadIdx.x; t < (ty + 2) * (T.tz + 2) * nx; t += blockDim.x) P[t] = 0.0;
+    __syncthreads();
+    for (int t = threadIdx.x; t < T.nrow * nx; t += blockDim.x) {
+        const int row = sort_div(T.magic_nx, t), i = t - row * nx, kl = sort_div(T.magic_ty, row), jl = row - kl * ty;
+        const long long c = (long long)(T.k0 + kl) * d.plane + (long long)(T.j0 + jl) * d.pitch + i + 1;
+        P[((kl + 1) * (ty + 2) + jl + 1) * nx + i] = SORT_OKP(c) ? T.A.p_hi[c] : 0.0;
+        B[t] = SORT_OKP(c) ? T.A.b[c] : 0.0f;
+    }
+    __syncthreads();
+}
+
+// e = 0 on the tile.
+__device__ __forceinline__ void sort_clear_e(const SorTile &T)
+{
     __syncthreads();
     float4 *E = sort_e(T, 0);
     for (int t = threadIdx.x; t < 2 * T.ncol; t += blockDim.x) E[t] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
+}
+
+// p_hi += e on the tile, e = 0; four slots (two cells each) in flight.
+__device__ __noinline__ void sort_fold()
+{
+    SorTile &T = sort_tile();
+    const PDims &d = T.A.d;
+    const int nx = d.nx, slots = (nx + 1) >> 1, ty = T.ty, G = T.G, ps = T.ps, e0 = T.e0, n = T.nrow * slots;
+    double *p_hi = T.A.p_hi;
+    const float *E0 = reinterpret_cast<const float *>(sort_e(T, 0));
+    const int other = 4 * T.ncol;
+    for (int t0 = threadIdx.x; t0 < n; t0 += 4 * blockDim.x) {
+        double pa[4], pb[4];
+        int at[4];  // element of p_hi (a grid that fits has fewer than 2^31)
+        float ea[4], eb[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const int t = t0 + m * blockDim.x;
+            at[m] = -1;
+            if (t < n) {
+                const int row = sort_div(T.magic_slots, t), s = t - row * slots;
+                const int kl = sort_div(T.magic_ty, row), jl = row - kl * ty, i = 2 * s + 1;
+                const int c = (int)((long long)(T.k0 + kl) * d.plane) + (T.j0 + jl) * d.pitch + i;
+                // cell i is of colour (i + j + k) & 1, cell i + 1 of the other (past the row's end: a pad slot, 0)
+                const int c0 = (i + T.j0 + jl + T.k0 + kl) & 1;
+                const int at_e = 4 * (e0 + kl * ps + jl * G) + s;
+                ea[m] = E0[at_e + (c0 ? other : 0)];
+                eb[m] = E0[at_e + (c0 ? 0 : other)];
+                pa[m] = SORT_OKP(c) ? p_hi[c] : 0.0;
+                pb[m] = SORT_OKP(c + 1) ? p_hi[c + 1] : 0.0;  // the ghost column at most
+                at[m] = c;
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            if (at[m] < 0) continue;
+            if (SORT_OKP(at[m])) p_hi[at[m]] = pa[m] + f64_from_f32(ea[m]);
+            if (eb[m] != 0.0f && SORT_OKP(at[m] + 1)) p_hi[at[m] + 1] = pb[m] + f64_from_f32(eb[m]);
+        }
+    }
+    sort_clear_e(T);
+}
+
+// The same for a register tile with its own copy of p: the rows on the rim
+// go to p_hi, where the neighbouring tiles read them, the others at the end.
+__device__ __noinline__ void sort_fold_copy()
+{
+    SorTile &T = sort_tile();
+    const PDims &d = T.A.d;
+    const int nx = d.nx, ty = T.ty, tz = T.tz, G = T.G, ps = T.ps, e0 = T.e0;
+    double *P = sort_p(T);
+    const float *E0 = reinterpret_cast<const float *>(sort_e(T, 0));
+    const int other = 4 * T.ncol;
+    for (int t = threadIdx.x; t < T.nrow * nx; t += blockDim.x) {
+        const int row = sort_div(T.magic_nx, t), i = t - row * nx + 1, kl = sort_div(T.magic_ty, row), jl = row - kl * ty;
+        const int c1 = (i + T.j0 + jl + T.k0 + kl) & 1;
+        const float e = E0[4 * (e0 + kl * ps + jl * G) + ((i - 1) >> 1) + (c1 ? other : 0)];
+        double *q = P + ((kl + 1) * (ty + 2) + jl + 1) * nx + i - 1;
+        const double p = *q + f64_from_f32(e);
+        *q = p;
+        const long long c = (long long)(T.k0 + kl) * d.plane + (long long)(T.j0 + jl) * d.pitch + i;
+        if ((jl == 0 || jl == ty - 1 || kl == 0 || kl == tz - 1) && SORT_OKP(c)) T.A.p_hi[c] = p;
+    }
+    sort_clear_e(T);
+}
+
+// The end of such a solve: the tile's p to p_hi.
+__device__ __noinline__ void sort_write_tile()
+{
+    SorTile &T = sort_tile();
+    const PDims &d = T.A.d;
+    const int nx = d.nx, ty = T.ty;
+    for (int t = threadIdx.x; t < T.nrow * nx; t += blockDim.x) {
+        const int row = sort_div(T.magic_nx, t), i = t - row * nx, kl = sort_div(T.magic_ty, row), jl = row - kl * ty;
+        const long long c = (long long)(T.k0 + kl) * d.plane + (long long)(T.j0 + jl) * d.pitch + i + 1;
+        if (SORT_OKP(c)) T.A.p_hi[c] = sort_p(T)[((kl + 1) * (ty + 2) + jl + 1) * nx + i];
+    }
 }
 
 // n_iter iterations of a tile of any size.  A half-sweep updates the rim
@@ -537,7 +678,7 @@ __device__ __noinline__ bool sort_sweeps(int n_iter)
     unsigned bits = 0;
     auto unit_at = [&](int u) {
         const int unit = min(u + lane, nunits - 1);
-        const int cb = sort_div_g(T.magic_g, unit), g = unit - cb * G;
+        const int cb = sort_div(T.magic_g, unit), g = unit - cb * G;
         const int seg = cb / njb, jl = 1 + 2 * (cb - seg * njb);
         // a segment is lseg planes long; the last one starts early enough to
         // end inside the tile and stores only its own planes
@@ -566,7 +707,7 @@ __device__ __noinline__ bool sort_sweeps(int n_iter)
         for (int n = 0; n < SORT_RB; ++n) {
             const int t = t0 + n * nthreads;
             if (t < T.nrim * G) {
-                const int row = sort_div_g(T.magic_g, t);
+                const int row = sort_div(T.magic_g, t);
                 r4[n] = load_r(rg, rim[row].roff + 4 * (t - row * G));
             }
         }
@@ -588,7 +729,7 @@ __device__ __noinline__ bool sort_sweeps(int n_iter)
             const int t = t0 + n * nthreads;
             vf[n] = zero4;
             if (far && t < T.nrim * G) {
-                const int row = sort_div_g(T.magic_g, t), g = t - row * G;
+                const int row = sort_div(T.magic_g, t), g = t - row * G;
                 const int fy = rim[row].fy, fz = rim[row].fz, f = fz >= 0 ? fz : fy;
                 if (f >= 0) vf[n] = load_r(eo, f + 4 * g);
             }
@@ -618,7 +759,7 @@ __device__ __noinline__ bool sort_sweeps(int n_iter)
                 for (int n = 0; n < SORT_RB; ++n) {
                     const int t = t0 + n * nthreads;
                     if (t < nitems) {
-                        const int row = sort_div_g(T.magic_g, t), g = t - row * G;
+                        const int row = sort_div(T.magic_g, t), g = t - row * G;
                         const int idx = rim[row].idx + g, off = rim[row].roff + 4 * g;
                         const unsigned w = rim[row].w;
                         const int kind = ((w ^ (unsigned)colour) & 1u) << 2 | (w & 2u) << 2 | (g == 0) | (g == G - 1) << 1;
@@ -776,8 +917,8 @@ __device__ __noinline__ bool sort_register_sweeps(int n_iter)
 #pragma unroll
     for (int m = 0; m < I; ++m) {
         const int t = tid + m * nthreads, tc = min(t, ngroups - 1);
-        const int row = sort_div_g(magic, tc), g = tc - row * G;
-        const int kl = row / ty, jl = row - kl * ty, k = T.k0 + kl;
+        const int row = sort_div(magic, tc), g = tc - row * G;
+        const int kl = sort_div(T.magic_ty, row), jl = row - kl * ty, k = T.k0 + kl;
         idx[m] = t < ngroups ? e0 + kl * ps + jl * G + g : -1;
         pub[m] = many && (jl == 0 || jl == ty - 1 || kl == 0 || kl == tz - 1) ? sort_rim_index(jl, kl, ty, tz) * G + g : -1;
         wrap[m] = T.py > 1 ? 0 : (jl == 0 ? ty * G : (jl == ty - 1 ? -ty * G : 0));
@@ -796,7 +937,7 @@ __device__ __noinline__ bool sort_register_sweeps(int n_iter)
         hsrc[m] = -1;
         hdst[m] = 0;
         if (t < nhalo) {
-            int row = sort_div_g(magic, t);
+            int row = sort_div(magic, t);
             const int g = t - row * G;
             if (row < 2 * tz) {
                 const int s = row >= tz, kl = row - s * tz;
@@ -875,6 +1016,12 @@ __device__ __noinline__ void sort_test(const SorTileRun &run, bool counting, int
         c.bb = bb;
     }
     c.rr = rr;
+    // far from the tolerance, and no prediction that needs the norm: no root, no division (a few us in FP64)
+    if (counting && !run.fixed && (run.chunk == 0 || run.chunk >= run.m) && isfinite(rr) && c.bb >= 1e-60 &&
+        rr > c.bb * run.tol2_above && c.iters < run.max_iter) {
+        c.next = run.chunk > 0 ? run.chunk : run.m;
+        return;
+    }
     const double rho = c.bb > 0.0 ? sqrt(rr / c.bb) : 0.0;
     c.rho = rho;
     const bool bad = !isfinite(rr) || !isfinite(c.bb) || !isfinite(rho);
@@ -911,6 +1058,8 @@ sor_solve_kernel(const __grid_constant__ SorTileArgs A, const __grid_constant__ 
         T.G = P.G;
         T.threads = P.threads;
         T.magic_g = P.magic_g;
+        T.magic_nx = sort_magic(A.d.nx);
+        T.magic_slots = sort_magic((A.d.nx + 1) >> 1);
         T.py = P.py;
         T.ntiles = P.py * P.pz;
         T.ta = blockIdx.x % P.py;
@@ -920,6 +1069,7 @@ sor_solve_kernel(const __grid_constant__ SorTileArgs A, const __grid_constant__ 
         T.k1 = (int)((long long)(T.tb + 1) * A.d.nz / P.pz);
         T.ty = (int)((long long)(T.ta + 1) * A.d.ny / P.py) - T.j0 + 1;
         T.tz = T.k1 - T.k0 + 1;
+        T.magic_ty = sort_magic(T.ty);
         T.nrow = T.ty * T.tz;
         // e of a register tile has a halo of one row on every side
         const int ety = I ? T.ty + 2 : T.ty;
@@ -929,7 +1079,7 @@ sor_solve_kernel(const __grid_constant__ SorTileArgs A, const __grid_constant__ 
         T.nrim = T.tz > 2 ? 2 * T.ty + (T.ty > 1 ? 2 : 1) * (T.tz - 2) : T.nrow;
         T.rim_half = A.rim_rows * P.G;
         T.barriers = 0;
-        T.epoch = A.sync[1];
+        T.epoch = A.sync[SORT_SYNC_EPOCH];
     }
     __syncthreads();
     SorTileDiag *diags = sort_diags(T, RSMEM);
@@ -959,46 +1109,82 @@ sor_solve_kernel(const __grid_constant__ SorTileArgs A, const __grid_constant__ 
     }
     __syncthreads();
 
-    bool ok, first = true;
-    int ran = 0;
-    for (;;) {
-        sort_residual<RSMEM>(first ? run.s_in : nullptr, !first && run.fixed ? run.s_out : nullptr, first);
-        ok = sort_grid_barrier();
-        if (!ok) break;
-        if (tid < 32) {
-            // the CTAs' partial sums in a fixed order, the same in every CTA
-            double rr = 0.0, bb = 0.0;
-            for (int q = tid; q < (int)gridDim.x; q += 32) {
-                rr += __ldcg(A.partials + 2 * q);
-                if (first) bb += __ldcg(A.partials + 2 * q + 1);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                rr += __shfl_down_sync(0xffffffffu, rr, o);
-                bb += __shfl_down_sync(0xffffffffu, bb, o);
-            }
-            if (tid == 0) sort_test(run, !first, ran, rr, bb);
+    // Checks as kernels of their own: run.n iterations, or with run.n < 0 those until the next check.
+    if (!A.plan.psm) {
+        int n = run.n;
+        if (n < 0) n = run.chunk * ((A.ctl->next + run.chunk - 1) / run.chunk);
+        if (RSMEM) sort_read_r();
+        __syncthreads();
+        bool ok;
+        if constexpr (I > 0) ok = sort_register_sweeps<I>(n);
+        else ok = sort_sweeps<RSMEM>(n);
+        if (ok) {
+            __syncthreads();
+            sort_fold();
+            if (I > 0) ok = sort_grid_barrier();  // every CTA has read the epoch
         }
-        __syncthreads();
-        ran = T.c.next;
-        if (ran == 0 && !(run.fixed && first)) break;  // a fixed count of 0 still forms the final residual
-        first = false;
-        if constexpr (I > 0) ok = sort_register_sweeps<I>(ran);
-        else ok = sort_sweeps<RSMEM>(ran);
-        if (!ok) break;
-        __syncthreads();
-        if (tid == 0) T.epoch += 2 * ran;
-        sort_fold();
-        ok = sort_grid_barrier();
-        if (!ok) break;
+        if (tid == 0) {
+            if (!ok) {
+                atomicCAS(&A.ctl->status, DEV_OK, DEV_TIMEOUT);
+                atomicAdd(A.sync + SORT_SYNC_EPOCH, 1u << 24);
+            } else if (blockIdx.x == 0) {
+                A.ctl->since = n;
+                if (I > 0) atomicAdd(A.sync + SORT_SYNC_EPOCH, 2u * n);
+            }
+        }
+        return;
     }
-    if (tid == 0) {
-        if (!ok) {
-            atomicCAS(&A.ctl->status, DEV_OK, DEV_TIMEOUT);
-            atomicAdd(A.sync + 1, 1u << 24);  // past every epoch that this solve may have published
-        } else if (blockIdx.x == 0) {
-            *A.ctl = T.c;
-            A.sync[1] = T.epoch;
+    if constexpr (I > 0) {
+        bool ok, first = true;
+        int ran = 0;
+        sort_read_tile();
+        for (;;) {
+            sort_residual(first ? run.s_in : nullptr, !first && run.fixed ? run.s_out : nullptr, first);
+            ok = sort_grid_barrier();
+            if (!ok) break;
+            if (tid < 32) {
+                // the CTAs' partial sums in a fixed order, the same in every CTA
+                double rr = 0.0, bb = 0.0;
+                for (int q0 = tid; q0 < (int)gridDim.x; q0 += 5 * 32) {
+                    double v[5];
+#pragma unroll
+                    for (int m = 0; m < 5; ++m) {
+                        const int q = q0 + 32 * m;
+                        v[m] = q < (int)gridDim.x ? __ldcg(A.partials + 2 * q) : 0.0;
+                    }
+#pragma unroll
+                    for (int m = 0; m < 5; ++m) rr += v[m];
+                }
+                if (first)
+                    for (int q = tid; q < (int)gridDim.x; q += 32) bb += __ldcg(A.partials + 2 * q + 1);
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    rr += __shfl_down_sync(0xffffffffu, rr, o);
+                    if (first) bb += __shfl_down_sync(0xffffffffu, bb, o);
+                }
+                if (tid == 0) sort_test(run, !first, ran, rr, bb);
+            }
+            __syncthreads();
+            ran = T.c.next;
+            if (ran == 0 && !(run.fixed && first)) break;  // a fixed count of 0 still forms the final residual
+            first = false;
+            ok = sort_register_sweeps<I>(ran);
+            if (!ok) break;
+            __syncthreads();
+            if (tid == 0) T.epoch += 2 * ran;
+            sort_fold_copy();
+            ok = sort_grid_barrier();
+            if (!ok) break;
+        }
+        if (ok) sort_write_tile();
+        if (tid == 0) {
+            if (!ok) {
+                atomicCAS(&A.ctl->status, DEV_OK, DEV_TIMEOUT);
+                atomicAdd(A.sync + SORT_SYNC_EPOCH, 1u << 24);  // past every epoch that this solve may have published
+            } else if (blockIdx.x == 0) {
+                *A.ctl = T.c;
+                A.sync[SORT_SYNC_EPOCH] = T.epoch;
+            }
         }
     }
 }
