@@ -16,12 +16,29 @@
 // the same on every launch shape.  FP32 is the fast path (sw_step); this
 // variant exists for precision: it is the method in FP64 end to end.
 //
+// What bounds it.  An FP64 instruction takes this GPU as long as 64 FP32 or
+// integer ones, so the kernels are written for few FP64 instructions (31 per
+// cell and step, against about 110 for the formulas as they stand) with the
+// same roundings:
+//   - the depth h = H + eta is formed once per cell and step and kept;
+//   - a face's flux is formed once, with its velocity (one of its two
+//     products is a zero);
+//   - comparisons are integer comparisons of the bit patterns;
+//   - a division by dx or dy is a product with the rounded reciprocal and
+//     one or two FMA corrections (s64_div), correctly rounded;
+//   - 1 - q n comes from a table of five values.
+// 700x501 cells: about 75 us per step with the formulas as they stand, 24 us so;
+// the FP64 pipe's floor for 31 instructions per cell is 17 us.
+//
 // Device layout: (ny + 2) rows of `pitch` doubles, cell (i, j) (1-based
-// interior, 0 and n + 1 the halo ring) at j * pitch + i; u[j][i] is the
-// east face of cell (i, j) (i = 0 .. nx), v[j][i] the north face
-// (j = 0 .. ny).  The halo ring of H and eta is 0, so it reads as dry.
+// interior, 0 and n + 1 the halo ring) at j * pitch + i; u[j][i] and F[j][i]
+// are the east face of cell (i, j) (i = 0 .. nx), v[j][i] and G[j][i] the
+// north face (j = 0 .. ny).  Walls and the halo ring stay 0 (h = 0 reads as
+// dry).
 #include <math.h>
+#include <stdint.h>
 #include <stdlib.h>
+#include <string.h>
 
 #include <algorithm>
 #include <new>
@@ -34,12 +51,14 @@ struct gbsw_sw64 {
     int pitch;
     cudaStream_t stream;
     double *H;                // (ny+2) x pitch
-    double *eta, *eta_new;    // state and the filtered elevation of the step
-    double *u, *v, *un, *vn;  // velocities and the predicted ones
+    double *eta, *u, *v;      // the state, updated in place
+    double *F, *G;            // fluxes through the east and north faces
+    double *h[2];             // depth H + eta at the start of the step ([cur]) and of the next one
     double *es;               // eta* of the step
+    int cur;
+    cudaGraphExec_t chunk[2]; // S64_CHUNK steps from h[0], h[1] as a graph
     double *partials, *result;
     double *h_result;         // pinned, 3 doubles
-    std::vector<double> h_H;  // host copy of H (interior, ny x nx) for the wet mask
 };
 
 namespace {
@@ -47,123 +66,176 @@ namespace {
 constexpr int S64_THREADS = 128;
 constexpr int S64_VOL_BLOCKS = 512;
 
+constexpr int S64_CHUNK = 16;  // steps per replayed graph (even: a chunk ends on the buffer it started from)
+
 struct S64Dev {
     int nx, ny, pitch;
     double gdt;   // g * dt
     double dx, dy, dt;
     double q;     // eps / 4
     double hmin;
+    double ydx, ydy;      // RN(1 / dx), RN(1 / dy)
+    int ndx, ndy;         // corrections that s64_div needs (0: plain division)
+    long long hmin_bits;  // of hmin (not negative)
+    double coef[5];       // RN(1 - RN(q n))
 };
 
-__device__ __forceinline__ bool s64_interior(const S64Dev &p, int i, int j)
-{
-    return i >= 1 && i <= p.nx && j >= 1 && j <= p.ny;
-}
+constexpr long long S64_INF = 0x7ff0000000000000LL;
 
-// Total depth H + eta of cell (i, j) at the start of the step; 0 off the grid.
-__device__ __forceinline__ double s64_depth(const S64Dev &p, const double *H, const double *eta, int i, int j)
+__device__ __forceinline__ bool s64_wet(const S64Dev &p, double h)  // h > hmin
 {
-    const long long c = (long long)j * p.pitch + i;
-    return s64_interior(p, i, j) ? __dadd_rn(H[c], eta[c]) : 0.0;
+    const long long b = __double_as_longlong(h);
+    return b > p.hmin_bits && b <= S64_INF;
 }
-
-__device__ __forceinline__ bool s64_wet(const S64Dev &p, const double *H, const double *eta, int i, int j)
+__device__ __forceinline__ bool s64_pos(double x)  // x > 0
 {
-    return s64_interior(p, i, j) && s64_depth(p, H, eta, i, j) > p.hmin;
+    const long long b = __double_as_longlong(x);
+    return b > 0 && b <= S64_INF;
+}
+__device__ __forceinline__ bool s64_neg(double x)  // x < 0
+{
+    return s64_pos(__longlong_as_double(__double_as_longlong(x) ^ (1LL << 63)));
+}
+__device__ __forceinline__ int s64_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// x / d rounded to nearest even, y = RN(1/d): q = RN(x y); if q is within one
+// unit in the last place, its remainder is exact in one FMA and q + r y,
+// rounded once, is the correctly rounded quotient (P. Markstein, "IA-64 and
+// Elementary Functions", Prentice Hall 2000, ch. 8).  q is off by less than
+// 1/2 unit (its own rounding) + 2 |1 - y d| 2^52 units, so n = 1 when
+// |1 - y d| <= 2^-54, else a second correction follows the first.  Exponents
+// at which a remainder could leave the normal range take the division.
+__device__ __forceinline__ double s64_div(double x, double d, double y, int n)
+{
+    if (n > 0 && (unsigned)(s64_exponent(x) - 200) < 1600u) {
+        double q = __dmul_rn(x, y);
+        q = __fma_rn(__fma_rn(-q, d, x), y, q);
+        if (n > 1) q = __fma_rn(__fma_rn(-q, d, x), y, q);
+        return q;
+    }
+    if ((__double_as_longlong(x) << 1) == 0) return x;  // a zero
+    return __ddiv_rn(x, d);
 }
 
 // Wet/dry face rule: a is the cell behind the face, b the cell ahead.
 __device__ __forceinline__ double s64_mask(double vel, bool wet_a, bool wet_b)
 {
-    if (wet_a && wet_b) return vel;
-    if (wet_a && vel > 0.0) return vel;
-    if (wet_b && vel < 0.0) return vel;
-    return 0.0;
+    return (wet_a && wet_b) || (wet_a && s64_pos(vel)) || (wet_b && s64_neg(vel)) ? vel : 0.0;
 }
 
-// Upwind volume flux through a face with velocity vel between cells a and b.
+// Upwind volume flux max(vel, 0) h_a + min(vel, 0) h_b through a face: one of
+// the products is a zero unless the other depth is not finite.
 __device__ __forceinline__ double s64_flux(double vel, double h_a, double h_b)
 {
-    const double up = vel > 0.0 ? vel : 0.0;
-    const double dn = vel < 0.0 ? vel : 0.0;
-    return __dadd_rn(__dmul_rn(up, h_a), __dmul_rn(dn, h_b));
+    const bool pos = s64_pos(vel), neg = s64_neg(vel);
+    if (s64_exponent(h_a) == 0x7ff || s64_exponent(h_b) == 0x7ff)
+        return __dadd_rn(__dmul_rn(pos ? vel : 0.0, h_a), __dmul_rn(neg ? vel : 0.0, h_b));
+    return pos || neg ? __dmul_rn(vel, pos ? h_a : h_b) : 0.0;
 }
 
-// Map 1 ("dyn", momentum): u' on faces (i = 0..nx, j = 1..ny) and v' on
-// faces (i = 1..nx, j = 0..ny); wall faces are 0.
-// Launch: grid (ceil((nx + 1) / S64_THREADS), ny + 1), block S64_THREADS.
-__global__ void __launch_bounds__(S64_THREADS)
-sw64_momentum_kernel(S64Dev p, const double *__restrict__ H, const double *__restrict__ eta,
-                     const double *__restrict__ u, const double *__restrict__ v, double *__restrict__ un,
-                     double *__restrict__ vn)
+// The kernels of a step follow one another as programmatic launches: each
+// may be scheduled while the one before drains, and reads nothing before
+// that one has completed.
+__device__ __forceinline__ void s64_wait()
 {
-    const int i = blockIdx.x * S64_THREADS + threadIdx.x;
-    const int j = blockIdx.y;
-    if (i > p.nx || j > p.ny) return;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// h = H + eta on the interior (the initial state).
+__global__ void __launch_bounds__(S64_THREADS)
+sw64_depth_kernel(S64Dev p, const double *H, const double *eta, double *h)
+{
+    const int i = blockIdx.x * S64_THREADS + threadIdx.x + 1, j = blockIdx.y + 1;
+    if (i > p.nx) return;
     const long long c = (long long)j * p.pitch + i;
-    if (j >= 1) {
-        double val = 0.0;
-        if (i >= 1 && i <= p.nx - 1) {
-            const double pred = __dsub_rn(u[c], __ddiv_rn(__dmul_rn(p.gdt, __dsub_rn(eta[c + 1], eta[c])), p.dx));
-            val = s64_mask(pred, s64_wet(p, H, eta, i, j), s64_wet(p, H, eta, i + 1, j));
-        }
-        un[c] = val;
+    h[c] = __dadd_rn(H[c], eta[c]);
+}
+
+// Map 1 ("dyn", momentum): u' and its flux on the east faces i = 1 .. nx-1,
+// v' and its flux on the north faces j = 1 .. ny-1 (wall faces stay 0).
+// Launch of the three maps: grid (ceil(nx / S64_THREADS), ny), block S64_THREADS.
+__global__ void __launch_bounds__(S64_THREADS)
+sw64_momentum_kernel(S64Dev p, const double *eta, const double *h, double *u, double *v, double *F, double *G)
+{
+    s64_wait();
+    const int i = blockIdx.x * S64_THREADS + threadIdx.x + 1, j = blockIdx.y + 1;
+    if (i > p.nx) return;
+    const long long c = (long long)j * p.pitch + i, n = c + p.pitch;
+    const double ec = eta[c], hc = h[c];
+    const bool wc = s64_wet(p, hc);
+    if (i < p.nx) {
+        const double he = h[c + 1];
+        const double pred = __dsub_rn(u[c], s64_div(__dmul_rn(p.gdt, __dsub_rn(eta[c + 1], ec)), p.dx, p.ydx, p.ndx));
+        const double vel = s64_mask(pred, wc, s64_wet(p, he));
+        u[c] = vel;
+        F[c] = s64_flux(vel, hc, he);
     }
-    if (i >= 1) {
-        double val = 0.0;
-        if (j >= 1 && j <= p.ny - 1) {
-            const double pred =
-                __dsub_rn(v[c], __ddiv_rn(__dmul_rn(p.gdt, __dsub_rn(eta[c + p.pitch], eta[c])), p.dy));
-            val = s64_mask(pred, s64_wet(p, H, eta, i, j), s64_wet(p, H, eta, i, j + 1));
-        }
-        vn[c] = val;
+    if (j < p.ny) {
+        const double hn = h[n];
+        const double pred = __dsub_rn(v[c], s64_div(__dmul_rn(p.gdt, __dsub_rn(eta[n], ec)), p.dy, p.ydy, p.ndy));
+        const double vel = s64_mask(pred, wc, s64_wet(p, hn));
+        v[c] = vel;
+        G[c] = s64_flux(vel, hc, hn);
     }
 }
 
 // Map 2 ("dyn", continuity): eta* on every interior cell.
-// Launch: grid (ceil(nx / S64_THREADS), ny), block S64_THREADS.
 __global__ void __launch_bounds__(S64_THREADS)
-sw64_continuity_kernel(S64Dev p, const double *__restrict__ H, const double *__restrict__ eta,
-                       const double *__restrict__ un, const double *__restrict__ vn, double *__restrict__ es)
+sw64_continuity_kernel(S64Dev p, const double *eta, const double *F, const double *G, double *es)
 {
-    const int i = blockIdx.x * S64_THREADS + threadIdx.x + 1;
-    const int j = blockIdx.y + 1;
+    s64_wait();
+    const int i = blockIdx.x * S64_THREADS + threadIdx.x + 1, j = blockIdx.y + 1;
     if (i > p.nx) return;
     const long long c = (long long)j * p.pitch + i;
-    const double hc = s64_depth(p, H, eta, i, j);
-    const double fe = s64_flux(un[c], hc, s64_depth(p, H, eta, i + 1, j));
-    const double fw = s64_flux(un[c - 1], s64_depth(p, H, eta, i - 1, j), hc);
-    const double gn = s64_flux(vn[c], hc, s64_depth(p, H, eta, i, j + 1));
-    const double gs = s64_flux(vn[c - p.pitch], s64_depth(p, H, eta, i, j - 1), hc);
-    const double div = __dadd_rn(__ddiv_rn(__dsub_rn(fe, fw), p.dx), __ddiv_rn(__dsub_rn(gn, gs), p.dy));
+    const double div = __dadd_rn(s64_div(__dsub_rn(F[c], F[c - 1]), p.dx, p.ydx, p.ndx),
+                                 s64_div(__dsub_rn(G[c], G[c - p.pitch]), p.dy, p.ydy, p.ndy));
     es[c] = __dsub_rn(eta[c], __dmul_rn(p.dt, div));
 }
 
 // Map 3 ("shapiro"): masked 5-point filter of eta* on wet cells (wet mask
-// of the start of the step).
-// Launch: grid (ceil(nx / S64_THREADS), ny), block S64_THREADS.
+// of the start of the step), and the depth of the next step.
 __global__ void __launch_bounds__(S64_THREADS)
-sw64_shapiro_kernel(S64Dev p, const double *__restrict__ H, const double *__restrict__ eta,
-                    const double *__restrict__ es, double *__restrict__ eta_new)
+sw64_shapiro_kernel(S64Dev p, const double *H, const double *h, const double *es, double *eta, double *h_next)
 {
-    const int i = blockIdx.x * S64_THREADS + threadIdx.x + 1;
-    const int j = blockIdx.y + 1;
+    s64_wait();
+    const int i = blockIdx.x * S64_THREADS + threadIdx.x + 1, j = blockIdx.y + 1;
     if (i > p.nx) return;
     const long long c = (long long)j * p.pitch + i;
-    if (!s64_wet(p, H, eta, i, j)) {
-        eta_new[c] = es[c];
-        return;
-    }
-    const int ni[4] = {i + 1, i - 1, i, i};
-    const int nj[4] = {j, j, j + 1, j - 1};
-    double count = 0.0, sum = 0.0;
+    double out = es[c];
+    if (s64_wet(p, h[c])) {
+        const long long nb[4] = {c + 1, c - 1, c + p.pitch, c - p.pitch};
+        int count = 0;
+        double sum = 0.0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-        if (s64_wet(p, H, eta, ni[k], nj[k])) {
-            count = __dadd_rn(count, 1.0);
-            sum = __dadd_rn(sum, es[(long long)nj[k] * p.pitch + ni[k]]);
-        }
-    eta_new[c] = __dadd_rn(__dmul_rn(__dsub_rn(1.0, __dmul_rn(p.q, count)), es[c]), __dmul_rn(p.q, sum));
+        for (int k = 0; k < 4; ++k)
+            if (s64_wet(p, h[nb[k]])) {
+                const double e = es[nb[k]];
+                sum = count ? __dadd_rn(sum, e) : e;
+                ++count;
+            }
+        const double coef = count == 4 ? p.coef[4] : count == 3 ? p.coef[3] : count == 2 ? p.coef[2]
+                          : count == 1 ? p.coef[1] : p.coef[0];
+        out = __dadd_rn(__dmul_rn(coef, out), __dmul_rn(p.q, sum));
+    }
+    eta[c] = out;
+    h_next[c] = __dadd_rn(H[c], out);
+}
+
+// Rows 0 .. rows-1 of `width` elements from `src` (row pitch p.pitch) packed into dst.
+__global__ void __launch_bounds__(S64_THREADS)
+sw64_pack_kernel(S64Dev p, const double *src, int width, double *dst)
+{
+    const int i = blockIdx.x * S64_THREADS + threadIdx.x, j = blockIdx.y;
+    if (i < width) dst[(size_t)j * width + i] = src[(size_t)j * p.pitch + i];
+}
+
+// Wet mask of the state as bytes.
+__global__ void __launch_bounds__(S64_THREADS)
+sw64_wet_kernel(S64Dev p, const double *h, uint8_t *wet)
+{
+    const int i = blockIdx.x * S64_THREADS + threadIdx.x, j = blockIdx.y;
+    if (i < p.nx) wet[(size_t)j * p.nx + i] = h[(size_t)(j + 1) * p.pitch + i + 1] > p.hmin;
 }
 
 // FP64 volume partials over rows b, b + S64_VOL_BLOCKS, ... (fixed order).
@@ -222,8 +294,63 @@ S64Dev s64_dev(const gbsw_sw64 *s)
     d.dy = s->p.dy;
     d.dt = s->p.dt;
     d.q = 0.25 * s->p.eps;
-    d.hmin = s->p.hmin;
+    d.hmin = s->p.hmin + 0.0;  // + 0.0: -0 as 0
+    memcpy(&d.hmin_bits, &d.hmin, sizeof(d.hmin));
+    for (int n = 0; n < 5; ++n) {
+        const volatile double qn = d.q * n;  // two roundings, as written
+        d.coef[n] = 1.0 - qn;
+    }
+    auto corrections = [](double x, double *y) {
+        *y = 1.0 / x;
+        if (!(x > 0x1p-100 && x < 0x1p100)) return 0;
+        return fabs(fma(-*y, x, 1.0)) <= 0x1p-54 ? 1 : 2;
+    };
+    d.ndx = corrections(d.dx, &d.ydx);
+    d.ndy = corrections(d.dy, &d.ydy);
     return d;
+}
+
+// One step from depth buffer a, on stream st; after: the launch before this one is another step's.
+cudaError_t s64_enqueue(const gbsw_sw64 *s, const S64Dev &d, int a, cudaStream_t st, bool after)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(gbsw::ceil_div(d.nx, S64_THREADS), d.ny);
+    cfg.blockDim = dim3(S64_THREADS);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = after ? attr : nullptr;
+    cfg.numAttrs = after ? 1 : 0;
+    const double *H = s->H, *h = s->h[a], *F = s->F, *G = s->G, *es = s->es, *eta = s->eta;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, sw64_momentum_kernel, d, eta, h, s->u, s->v, s->F, s->G);
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, sw64_continuity_kernel, d, eta, F, G, s->es);
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, sw64_shapiro_kernel, d, H, h, es, s->eta, s->h[1 - a]);
+    return e;
+}
+
+// The graph of S64_CHUNK steps from depth buffer a (captured on a private stream).
+cudaError_t s64_chunk(gbsw_sw64 *s, const S64Dev &d, int a)
+{
+    if (s->chunk[a]) return cudaSuccess;
+    cudaStream_t cs = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    cudaGraph_t g = nullptr;
+    e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        cudaError_t el = cudaSuccess;
+        for (int k = 0; k < S64_CHUNK && el == cudaSuccess; ++k) el = s64_enqueue(s, d, (a + k) & 1, cs, k > 0);
+        e = cudaStreamEndCapture(cs, &g);
+        if (e == cudaSuccess) e = el;
+    }
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&s->chunk[a], g, 0);
+    if (g) cudaGraphDestroy(g);
+    cudaStreamDestroy(cs);
+    if (e != cudaSuccess) s->chunk[a] = nullptr;
+    return e;
 }
 
 }  // namespace
@@ -235,7 +362,10 @@ extern "C" {
 void sw64_destroy(gbsw_sw64 *s)
 {
     if (!s) return;
-    double *bufs[] = {s->H, s->eta, s->eta_new, s->u, s->v, s->un, s->vn, s->es, s->partials, s->result};
+    cudaStreamSynchronize(s->stream);
+    for (cudaGraphExec_t g : s->chunk)
+        if (g) cudaGraphExecDestroy(g);
+    double *bufs[] = {s->H, s->eta, s->u, s->v, s->F, s->G, s->h[0], s->h[1], s->es, s->partials, s->result};
     for (double *b : bufs) cudaFree(b);
     if (s->h_result) cudaFreeHost(s->h_result);
     delete s;
@@ -267,9 +397,8 @@ gbsw_status sw64_create(const gbsw_sw_params *params, const double *H, const dou
     s->p = P;
     s->pitch = (int)round_up((size_t)P.nx + 2, 16);
     s->stream = (cudaStream_t)stream;
-    s->h_H.assign(H, H + n);
     const size_t bytes = (size_t)s->pitch * (size_t)(P.ny + 2) * sizeof(double);
-    double **fields[] = {&s->H, &s->eta, &s->eta_new, &s->u, &s->v, &s->un, &s->vn, &s->es};
+    double **fields[] = {&s->H, &s->eta, &s->u, &s->v, &s->F, &s->G, &s->h[0], &s->h[1], &s->es};
     for (double **f : fields) {
         cudaError_t err = cudaMalloc((void **)f, bytes);
         if (err == cudaSuccess) err = cudaMemsetAsync(*f, 0, bytes, s->stream);
@@ -288,6 +417,11 @@ gbsw_status sw64_create(const gbsw_sw_params *params, const double *H, const dou
         err = cudaMemcpy2DAsync(s->H + s->pitch + 1, dp, H, hp, hp, P.ny, cudaMemcpyHostToDevice, s->stream);
     if (err == cudaSuccess)
         err = cudaMemcpy2DAsync(s->eta + s->pitch + 1, dp, e.data(), hp, hp, P.ny, cudaMemcpyHostToDevice, s->stream);
+    if (err == cudaSuccess) {
+        const dim3 g(ceil_div(P.nx, S64_THREADS), P.ny);
+        sw64_depth_kernel<<<g, S64_THREADS, 0, s->stream>>>(s64_dev(s), s->H, s->eta, s->h[0]);
+        err = cudaGetLastError();
+    }
     if (err == cudaSuccess) err = cudaStreamSynchronize(s->stream);
     if (err != cudaSuccess) {
         record_cuda_error(err, "sw64_create", __FILE__, __LINE__);
@@ -303,17 +437,20 @@ gbsw_status sw64_step(gbsw_sw64 *s, int nsteps)
     gbsw::NvtxRange nvtx_range("sw64_step");
     if (!s || nsteps < 0) return GBSW_ERR_ARG;
     const S64Dev d = s64_dev(s);
-    const dim3 gf(ceil_div(d.nx + 1, S64_THREADS), d.ny + 1), gc(ceil_div(d.nx, S64_THREADS), d.ny);
-    for (int k = 0; k < nsteps; ++k) {
-        sw64_momentum_kernel<<<gf, S64_THREADS, 0, s->stream>>>(d, s->H, s->eta, s->u, s->v, s->un, s->vn);
-        sw64_continuity_kernel<<<gc, S64_THREADS, 0, s->stream>>>(d, s->H, s->eta, s->un, s->vn, s->es);
-        sw64_shapiro_kernel<<<gc, S64_THREADS, 0, s->stream>>>(d, s->H, s->eta, s->es, s->eta_new);
-        // update: eta <- eta+, u <- u', v <- v'
-        std::swap(s->eta, s->eta_new);
-        std::swap(s->u, s->un);
-        std::swap(s->v, s->vn);
+    int left = nsteps;
+    cudaError_t e = cudaSuccess;
+    for (; left >= S64_CHUNK && e == cudaSuccess; left -= S64_CHUNK) {
+        e = s64_chunk(s, d, s->cur);
+        if (e == cudaSuccess) e = cudaGraphLaunch(s->chunk[s->cur], s->stream);
     }
-    GBSW_LAUNCH_CHECK();
+    for (int k = 0; k < left && e == cudaSuccess; ++k) {
+        e = s64_enqueue(s, d, s->cur, s->stream, k > 0);
+        s->cur = 1 - s->cur;
+    }
+    if (e != cudaSuccess) {
+        record_cuda_error(e, "sw64_step", __FILE__, __LINE__);
+        return GBSW_ERR_CUDA;
+    }
     return GBSW_OK;
 }
 
@@ -335,23 +472,30 @@ gbsw_status sw64_get_state(gbsw_sw64 *s, double *eta, double *u, double *v, uint
 {
     if (!s) return GBSW_ERR_ARG;
     const int nx = s->p.nx, ny = s->p.ny;
-    const size_t dp = (size_t)s->pitch * sizeof(double);
-    std::vector<double> e;
-    if (eta || wet) {
-        e.resize((size_t)nx * ny);
-        GBSW_CUDA_TRY(cudaMemcpy2DAsync(e.data(), nx * sizeof(double), s->eta + s->pitch + 1, dp,
-                                        nx * sizeof(double), ny, cudaMemcpyDeviceToHost, s->stream));
+    // Each field is packed on the device (into es, which the next step writes
+    // anew) and copied in one piece: a pitched copy into pageable memory goes
+    // row by row.
+    const S64Dev d = s64_dev(s);
+    auto copy = [&](double *dst, const double *src, int width, int rows) -> gbsw_status {
+        const dim3 g(ceil_div(width, S64_THREADS), rows);
+        sw64_pack_kernel<<<g, S64_THREADS, 0, s->stream>>>(d, src, width, s->es);
+        GBSW_LAUNCH_CHECK();
+        GBSW_CUDA_TRY(cudaMemcpyAsync(dst, s->es, (size_t)width * rows * sizeof(double), cudaMemcpyDeviceToHost,
+                                      s->stream));
+        return GBSW_OK;
+    };
+    gbsw_status st = GBSW_OK;
+    if (eta) st = copy(eta, s->eta + s->pitch + 1, nx, ny);
+    if (u && st == GBSW_OK) st = copy(u, s->u + s->pitch, nx + 1, ny);  // east faces i = 0..nx of rows 1..ny
+    if (v && st == GBSW_OK) st = copy(v, s->v + 1, nx, ny + 1);         // north faces j = 0..ny of columns 1..nx
+    if (st != GBSW_OK) return st;
+    if (wet) {
+        const dim3 g(ceil_div(nx, S64_THREADS), ny);
+        sw64_wet_kernel<<<g, S64_THREADS, 0, s->stream>>>(d, s->h[s->cur], (uint8_t *)s->es);
+        GBSW_LAUNCH_CHECK();
+        GBSW_CUDA_TRY(cudaMemcpyAsync(wet, s->es, (size_t)nx * ny, cudaMemcpyDeviceToHost, s->stream));
     }
-    if (u)  // east faces i = 0..nx of rows 1..ny
-        GBSW_CUDA_TRY(cudaMemcpy2DAsync(u, (nx + 1) * sizeof(double), s->u + s->pitch, dp, (nx + 1) * sizeof(double),
-                                        ny, cudaMemcpyDeviceToHost, s->stream));
-    if (v)  // north faces j = 0..ny of columns 1..nx
-        GBSW_CUDA_TRY(cudaMemcpy2DAsync(v, nx * sizeof(double), s->v + 1, dp, nx * sizeof(double), ny + 1,
-                                        cudaMemcpyDeviceToHost, s->stream));
     GBSW_CUDA_TRY(cudaStreamSynchronize(s->stream));
-    if (eta) std::copy(e.begin(), e.end(), eta);
-    if (wet)
-        for (size_t k = 0; k < e.size(); ++k) wet[k] = (uint8_t)(s->h_H[k] + e[k] > s->p.hmin);
     return GBSW_OK;
 }
 
