@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "sw_chip.cuh"
 #include "sw_kernels.cuh"
 #include "sw_stream.cuh"
 #include "sw_tile.cuh"
@@ -100,6 +101,12 @@ struct gbsw_sw {
     double *result;         // 3 doubles on the device
     double *h_result;       // 3 doubles, pinned host
     uint8_t *wet;           // ny*nx bytes, staging for sw_get_state
+    SWChipPlan chip;        // automatic tiling of a grid that fits on the chip (cx = 0: it does not)
+    uint4 *pub;             // 2 ny*nx published cells
+    unsigned epoch;         // exchanges so far
+    int *status;            // device status word of the chip kernel
+    int *h_status;          // pinned copy
+    bool status_due;        // a chip launch has been enqueued since the status was last read
 };
 
 namespace {
@@ -257,6 +264,124 @@ cudaError_t launch_from(const gbsw_sw *s, int T, int rows, int a, cudaStream_t s
     }
 }
 
+const void *chip_kernel(int per)
+{
+    switch (per) {
+    case 1: return (const void *)sw_chip_kernel<1>;
+    case 2: return (const void *)sw_chip_kernel<2>;
+    case 4: return (const void *)sw_chip_kernel<4>;
+    case 6: return (const void *)sw_chip_kernel<6>;
+    case 8: return (const void *)sw_chip_kernel<8>;
+    case 12: return (const void *)sw_chip_kernel<12>;
+    default: return (const void *)sw_chip_kernel<16>;
+    }
+}
+
+size_t chip_smem(int per) { return ((size_t)SWC_ARRAYS * per * SWC_THREADS + 2 * SWC_GUARD) * sizeof(float); }
+
+// The cut of the grid for sw_chip_kernel: of all tiles and depths T that fit
+// the one with the least estimated cycles per step: 2000 for an exchange (none
+// with one tile), and per step 350 of latency and 330 for each cell of a
+// thread's region (16 warps of about 80 instructions on four schedulers).
+SWChipPlan chip_plan(int nx, int ny)
+{
+    SWChipPlan best{};
+    int dev = 0, coop = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) {
+        cudaGetLastError();
+        return best;
+    }
+    const int pers[] = {1, 2, 4, 6, 8, 12, 16};
+    const int sms = sm_count();
+    double best_cost = 0.0;
+    for (int T = 1; T <= SWC_MAX_T; ++T)
+        for (int cx = 1; cx <= std::min(sms, nx); ++cx) {
+            const int tw = ceil_div(nx, cx);
+            if (ceil_div(nx, tw) != cx) continue;  // the same tiles as with fewer columns
+            for (int cy = 1; cy <= std::min(sms / cx, ny); ++cy) {
+                const int th = ceil_div(ny, cy);
+                if (ceil_div(ny, th) != cy) continue;
+                const long long cells = (long long)(tw + 4 * T) * (th + 4 * T);
+                if (cells > 16 * SWC_THREADS || tw + 4 * T >= SWC_GUARD) continue;
+                int per = 16;
+                for (int c : pers)
+                    if (cells <= (long long)c * SWC_THREADS) {
+                        per = c;
+                        break;
+                    }
+                const double cost = (cx * cy > 1 ? 2000.0 / T : 0.0) + 350.0 + 330.0 * per;
+                if (best.cx && cost >= best_cost) continue;
+                best_cost = cost;
+                best = SWChipPlan{cx, cy, tw, th, T, per};
+            }
+        }
+    if (!best.cx) return best;
+    const void *fn = chip_kernel(best.per);
+    int per_sm = 0;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chip_smem(best.per)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, SWC_THREADS, chip_smem(best.per)) != cudaSuccess ||
+        per_sm < 1) {
+        cudaGetLastError();
+        best.cx = 0;
+    }
+    return best;
+}
+
+// nsteps steps as one launch of the chip kernel.
+gbsw_status run_chip(gbsw_sw *s, int nsteps)
+{
+    if (nsteps == 0) return GBSW_OK;
+    const int a = s->cur, b = 1 - a;
+    unsigned epoch = s->epoch;
+    const float *H = s->H, *ei = s->eta[a], *ui = s->u[a], *vi = s->v[a];
+    void *args[] = {&s->d, &s->chip, &nsteps, &epoch, &s->pub, &s->status, &H, &ei, &ui, &vi, &s->eta[b], &s->u[b], &s->v[b]};
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(s->chip.cx, s->chip.cy);
+    cfg.blockDim = dim3(SWC_THREADS);
+    cfg.dynamicSmemBytes = chip_smem(s->chip.per);
+    cfg.stream = s->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    GBSW_CUDA_TRY(cudaLaunchKernelExC(&cfg, chip_kernel(s->chip.per), args));
+    s->epoch += (nsteps - 1) / s->chip.T;  // exchanges of this launch
+    s->cur = b;
+    s->status_due = true;
+    return GBSW_OK;
+}
+
+// Enqueue the read of the chip kernel's status word before a synchronisation, and judge it after.
+gbsw_status status_read(gbsw_sw *s)
+{
+    if (s->status_due)
+        GBSW_CUDA_TRY(cudaMemcpyAsync(s->h_status, s->status, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+    return GBSW_OK;
+}
+
+gbsw_status status_judge(gbsw_sw *s)
+{
+    if (!s->status_due) return GBSW_OK;
+    s->status_due = false;
+    const gbsw_status st = dev_status_to_gbsw(*s->h_status);
+    if (st != GBSW_OK) cudaMemsetAsync(s->status, 0, sizeof(int), s->stream);
+    return st;
+}
+
+// True if the context's stream is being captured: the chip kernel's exchange
+// numbers are launch arguments that a replay would repeat.
+bool capturing(const gbsw_sw *s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s->stream, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
 int auto_blocking(const gbsw_sw *) { return 3; }
 
 int tiling_T(const gbsw_sw *s) { return s->blocking > 0 ? s->blocking : auto_blocking(s); }
@@ -399,13 +524,27 @@ gbsw_status sw_create(const gbsw_sw_params *params, const double *H, const doubl
     SW_ALLOC(s->partials, SW_VOL_BLOCKS * 3 * sizeof(double));
     SW_ALLOC(s->result, 3 * sizeof(double));
     SW_ALLOC(s->wet, n);
+    SW_ALLOC(s->status, sizeof(int));
 #undef SW_ALLOC
-    if (cudaMallocHost((void **)&s->h_result, 3 * sizeof(double)) != cudaSuccess) return fail(GBSW_ERR_OOM);
+    if (cudaMallocHost((void **)&s->h_result, 4 * sizeof(double)) != cudaSuccess) return fail(GBSW_ERR_OOM);
+    s->h_status = (int *)(s->h_result + 3);
+    s->chip = chip_plan(P.nx, P.ny);
+    if (s->chip.cx * s->chip.cy > 1) {
+        const size_t pb = 2 * n * sizeof(uint4);
+        if (cudaMalloc((void **)&s->pub, pb) != cudaSuccess) {  // no room: the launches need none
+            cudaGetLastError();
+            s->pub = nullptr;
+            s->chip.cx = 0;
+        } else if (cudaMemsetAsync(s->pub, 0, pb, s->stream) != cudaSuccess) {
+            return fail(GBSW_ERR_CUDA);
+        }
+    }
 
     cudaError_t e = cudaSuccess;
     float *all[7] = {s->H, s->eta[0], s->eta[1], s->u[0], s->u[1], s->v[0], s->v[1]};
     for (float *ptr : all)
         if (e == cudaSuccess) e = cudaMemsetAsync(ptr, 0, bytes, s->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s->status, 0, sizeof(int), s->stream);
     const size_t dp = (size_t)s->d.pitch * sizeof(float), hp = (size_t)P.nx * sizeof(float);
     if (e == cudaSuccess)
         e = cudaMemcpy2DAsync(s->H, dp, h32.data(), hp, hp, P.ny, cudaMemcpyHostToDevice, s->stream);
@@ -442,6 +581,7 @@ gbsw_status sw_step(gbsw_sw *s, int nsteps)
 {
     gbsw::NvtxRange nvtx_range("sw_step");
     if (!s || nsteps < 0) return GBSW_ERR_ARG;
+    if (s->blocking == 0 && s->rows == 0 && s->chip.cx && !capturing(s)) return run_chip(s, nsteps);
     const int T = tiling_T(s);
     return run_steps(s, nsteps, T, tiling_rows(s, T));
 }
@@ -456,6 +596,7 @@ gbsw_status sw_autotune(gbsw_sw *s, int trial_steps, int *T_out, int *rows_out)
     gbsw_status st = GBSW_OK;
     int bestT = tiling_T(s), best_rows = tiling_rows(s, bestT);
     float best = INFINITY;
+    bool automatic = false;  // the automatic tiling (the chip kernel) is the fastest
     const int c0 = s->cur;
     do {
         bool ok = true;
@@ -507,6 +648,18 @@ gbsw_status sw_autotune(gbsw_sw *s, int trial_steps, int *T_out, int *rows_out)
                 }
             }
         }
+        if (st == GBSW_OK && s->chip.cx) {
+            float ms = 0.0f;
+            if ((st = run_chip(s, trial_steps)) == GBSW_OK) {
+                cudaEventRecord(e0, s->stream);
+                st = run_chip(s, trial_steps);
+                cudaEventRecord(e1, s->stream);
+            }
+            if (st == GBSW_OK &&
+                (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
+                st = GBSW_ERR_CUDA;
+            automatic = st == GBSW_OK && ms / trial_steps < best;
+        }
         // restore the state: results do not depend on the tiling, so the
         // trials leave no trace
         const int c = s->cur;
@@ -520,8 +673,8 @@ gbsw_status sw_autotune(gbsw_sw *s, int trial_steps, int *T_out, int *rows_out)
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     if (st != GBSW_OK) return st;
-    s->blocking = bestT;
-    s->rows = best_rows;
+    s->blocking = automatic ? 0 : bestT;
+    s->rows = automatic ? 0 : best_rows;
     if (T_out) *T_out = bestT;
     if (rows_out) *rows_out = best_rows;
     return GBSW_OK;
@@ -538,7 +691,10 @@ gbsw_status sw_volume(gbsw_sw *s, double *volume, double *wet_volume)
                                                                s->p.dx * s->p.dy, s->result);
     GBSW_LAUNCH_CHECK();
     GBSW_CUDA_TRY(cudaMemcpyAsync(s->h_result, s->result, 3 * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
+    gbsw_status st = status_read(s);
+    if (st != GBSW_OK) return st;
     GBSW_CUDA_TRY(cudaStreamSynchronize(s->stream));
+    if ((st = status_judge(s)) != GBSW_OK) return st;
     if (volume) *volume = s->h_result[0];
     if (wet_volume) *wet_volume = s->h_result[1];
     return s->h_result[2] != 0.0 ? GBSW_ERR_NONFINITE : GBSW_OK;
@@ -564,7 +720,10 @@ gbsw_status sw_get_state(gbsw_sw *s, float *eta, float *u, float *v, uint8_t *we
         GBSW_LAUNCH_CHECK();
         GBSW_CUDA_TRY(cudaMemcpyAsync(wet, s->wet, (size_t)nx * ny, cudaMemcpyDeviceToHost, s->stream));
     }
+    gbsw_status st = status_read(s);
+    if (st != GBSW_OK) return st;
     GBSW_CUDA_TRY(cudaStreamSynchronize(s->stream));
+    if ((st = status_judge(s)) != GBSW_OK) return st;
     if (u)
         for (int j = 0; j < ny; ++j) u[(size_t)j * (nx + 1)] = 0.0f;
     if (v)
@@ -609,6 +768,8 @@ void sw_destroy(gbsw_sw *s)
     cudaFree(s->partials);
     cudaFree(s->result);
     cudaFree(s->wet);
+    cudaFree(s->pub);
+    cudaFree(s->status);
     if (s->h_result) cudaFreeHost(s->h_result);
     free(s);
 }
