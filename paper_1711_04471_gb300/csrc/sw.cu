@@ -264,25 +264,24 @@ cudaError_t launch_from(const gbsw_sw *s, int T, int rows, int a, cudaStream_t s
     }
 }
 
-const void *chip_kernel(int per)
+template <int PER>
+const void *chip_kernel_of(int per)
 {
-    switch (per) {
-    case 1: return (const void *)sw_chip_kernel<1>;
-    case 2: return (const void *)sw_chip_kernel<2>;
-    case 4: return (const void *)sw_chip_kernel<4>;
-    case 6: return (const void *)sw_chip_kernel<6>;
-    case 8: return (const void *)sw_chip_kernel<8>;
-    case 12: return (const void *)sw_chip_kernel<12>;
-    default: return (const void *)sw_chip_kernel<16>;
+    if constexpr (PER < SWC_MAX_PER) {
+        if (per != PER) return chip_kernel_of<PER + 1>(per);
     }
+    return (const void *)sw_chip_kernel<PER>;
 }
+
+// The kernel for `per` cells per thread (1 .. SWC_MAX_PER).
+const void *chip_kernel(int per) { return chip_kernel_of<1>(per); }
 
 size_t chip_smem(int per) { return ((size_t)SWC_ARRAYS * per * SWC_THREADS + 2 * SWC_GUARD) * sizeof(float); }
 
 // The cut of the grid for sw_chip_kernel: of all tiles and depths T that fit
 // the one with the least estimated cycles per step: 2000 for an exchange (none
-// with one tile), and per step 350 of latency and 330 for each cell of a
-// thread's region (16 warps of about 80 instructions on four schedulers).
+// with one tile), and per step 300 of latency and 650 for each cell of a
+// thread (measured: 500x500 4200 cycles, 700x700 7400).
 SWChipPlan chip_plan(int nx, int ny)
 {
     SWChipPlan best{};
@@ -292,7 +291,6 @@ SWChipPlan chip_plan(int nx, int ny)
         cudaGetLastError();
         return best;
     }
-    const int pers[] = {1, 2, 4, 6, 8, 12, 16};
     const int sms = sm_count();
     double best_cost = 0.0;
     for (int T = 1; T <= SWC_MAX_T; ++T)
@@ -303,14 +301,9 @@ SWChipPlan chip_plan(int nx, int ny)
                 const int th = ceil_div(ny, cy);
                 if (ceil_div(ny, th) != cy) continue;
                 const long long cells = (long long)(tw + 4 * T) * (th + 4 * T);
-                if (cells > 16 * SWC_THREADS || tw + 4 * T >= SWC_GUARD) continue;
-                int per = 16;
-                for (int c : pers)
-                    if (cells <= (long long)c * SWC_THREADS) {
-                        per = c;
-                        break;
-                    }
-                const double cost = (cx * cy > 1 ? 2000.0 / T : 0.0) + 350.0 + 330.0 * per;
+                const int per = ceil_div(cells, SWC_THREADS);
+                if (per > SWC_MAX_PER || tw + 4 * T >= SWC_GUARD) continue;
+                const double cost = (cx * cy > 1 ? 2000.0 / T : 0.0) + 300.0 + 650.0 * per;
                 if (best.cx && cost >= best_cost) continue;
                 best_cost = cost;
                 best = SWChipPlan{cx, cy, tw, th, T, per};

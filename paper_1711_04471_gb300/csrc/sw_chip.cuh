@@ -14,15 +14,18 @@
 // neighbours, which they wrote after reading its exchange k.
 //
 // Each step is three barrier-separated phases over the region, as in
-// sw_tile_kernel, with fewer operations: a cell publishes its filtered
-// elevation already multiplied by its wet mask, and counts its wet
-// neighbours where it has just read their depths.  Every rounding is the
-// streaming kernel's, so the states are bitwise the same.
+// sw_tile_kernel, with fewer operations: a face's flux is formed once, with
+// its velocity; a cell publishes its filtered elevation already multiplied
+// by its wet mask, beside the mask; and the phases are branch-free, so that
+// a thread's cells overlap.  Every rounding is the streaming kernel's, so
+// the states are bitwise the same.  (Four cells of a row per thread with
+// packed FP32 operations was slower: 3.2 us per step at 500x500.)
 //
 // What bounds it: the way of a word from SM to SM (about 1 us per exchange)
-// on small grids, the issue slots of the phases on large ones.  us per step,
-// the kernel that the autotuner chose before, this one: 100x100 1.19, 0.66;
-// 500x500 2.55, 2.20; 1000x1000 8.9, 7.5 (untuned, the launches took 10 us and more).
+// on small grids, the issue slots and shared-memory wavefronts of the phases
+// on large ones.  us per step, the kernel that the autotuner chose before,
+// this one: 100x100 1.19, 0.65; 500x500 2.55, 2.05; 700x700 5.0, 3.6;
+// 1000x1000 8.9, 7.2 (untuned, the launches took 10 us and more).
 #pragma once
 
 #include "sw_kernels.cuh"
@@ -32,7 +35,8 @@ namespace gbsw {
 constexpr int SWC_THREADS = 512;
 constexpr int SWC_MAX_T = 4;
 constexpr int SWC_GUARD = 2048;        // most columns of a region
-constexpr int SWC_ARRAYS = 5;          // shared FP32 arrays of a region
+constexpr int SWC_ARRAYS = 6;          // shared FP32 arrays of a region
+constexpr int SWC_MAX_PER = 16;        // cells per thread at most
 constexpr long long SWC_WAIT_CYCLES = 4000000000LL;
 
 // How a grid is cut: cx x cy tiles of tw x th cells (the last ones smaller),
@@ -57,10 +61,22 @@ __device__ __forceinline__ void swc_store(uint4 *p, float a, float b, float c, u
                  ::"l"(p), "l"(lo), "l"(hi) : "memory");
 }
 
+// Velocity of a face and its parts that carry flux: vel as predicted, the
+// cells behind and ahead wet (both false: a wall).  The masked velocity's
+// positive part needs the cell behind to be wet, its negative part the cell
+// ahead (the rule of sw_face_mask).
+__device__ __forceinline__ float swc_face(float vel, bool wet_b, bool wet_a, float *pos, float *neg)
+{
+    *pos = wet_b ? fmaxf(vel, 0.0f) : 0.0f;
+    *neg = wet_a ? fminf(vel, 0.0f) : 0.0f;
+    return wet_b && wet_a ? vel : __fadd_rn(*pos, *neg);
+}
+
 // nsteps steps from (eta_in, u_in, v_in) to (eta_out, u_out, v_out).  pub:
-// two arrays of ny x nx words (NULL with a single tile); epoch0: number of the last exchange of
-// earlier launches.  Cooperative launch: grid (cx, cy), block SWC_THREADS,
-// SWC_ARRAYS x PER x SWC_THREADS + 2 SWC_GUARD floats of dynamic shared memory.
+// two arrays of ny x nx words (NULL with a single tile); epoch0: number of
+// the last exchange of earlier launches.  Cooperative launch: grid (cx, cy),
+// block SWC_THREADS, SWC_ARRAYS x PER x SWC_THREADS + 2 SWC_GUARD floats of
+// dynamic shared memory.
 template <int PER>
 __global__ void __launch_bounds__(SWC_THREADS, 1)
 sw_chip_kernel(SWDev p, SWChipPlan P, int nsteps, unsigned epoch0, uint4 *pub, int *status,
@@ -69,10 +85,14 @@ sw_chip_kernel(SWDev p, SWChipPlan P, int nsteps, unsigned epoch0, uint4 *pub, i
                float *__restrict__ v_out)
 {
     constexpr int NC = PER * SWC_THREADS;
+    constexpr bool FREG = PER <= 7;  // a cell's own fluxes wait in registers, else they are read back
     extern __shared__ float swc_smem[];
-    // the arrays, with a row's worth of slack on both sides (reads of the rows
-    // below the first and above the last array's end)
-    float *const e = swc_smem + SWC_GUARD, *const hh = e + NC, *const uu = hh + NC, *const vv = uu + NC, *const we = vv + NC;
+    // depth and elevation; fluxes through the east and north faces; masked
+    // eta* and wet mask in pairs, and a row's worth of slack.  The rows below an
+    // array's first and above its last one are read from what lies there (the
+    // array before, the array after, the slack) and not used.
+    float *const hh = swc_smem, *const e = hh + NC, *const ff = e + NC, *const gg = ff + NC;
+    float2 *const we = reinterpret_cast<float2 *>(gg + NC);
     const int tid = threadIdx.x, T = P.T, halo = 2 * T;
     const int x0 = blockIdx.x * P.tw - halo, y0 = blockIdx.y * P.th - halo;
     const int tw = min(P.tw, p.nx - (int)blockIdx.x * P.tw), th = min(P.th, p.ny - (int)blockIdx.y * P.th);
@@ -82,10 +102,8 @@ sw_chip_kernel(SWDev p, SWChipPlan P, int nsteps, unsigned epoch0, uint4 *pub, i
     (void)extent;
     (void)words;
     constexpr unsigned F_CELL = 1u, F_EAST = 2u, F_NORTH = 4u, F_INNER = 8u, F_STORE = 16u, F_HALO = 32u, F_PUB = 64u;
-    // 1 - q x (wet neighbours) waits in a register, or, where registers are
-    // short, the count does in the flags (bits 8 ..)
-    constexpr bool COEF = PER < 12;
-    float re[PER], ru[PER], rv[PER], rH[PER], rc[COEF ? PER : 1];
+    constexpr unsigned F_WET = 128u;  // wet at the start of the step
+    float re[PER], ru[PER], rv[PER], rH[PER], rf[FREG ? PER : 1], rg[FREG ? PER : 1];
     unsigned m[PER];
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
@@ -93,7 +111,6 @@ sw_chip_kernel(SWDev p, SWChipPlan P, int nsteps, unsigned epoch0, uint4 *pub, i
         const int gx = x0 + lx, gy = y0 + ly;
         unsigned f = 0;
         re[k] = ru[k] = rv[k] = rH[k] = 0.0f;
-        if (COEF) rc[COEF ? k : 0] = 1.0f;
         if (ly < LH) {
             f = F_CELL;
             if (lx + 1 < LW && gx >= 0 && gx < p.nx - 1) f |= F_EAST;
@@ -121,51 +138,49 @@ sw_chip_kernel(SWDev p, SWChipPlan P, int nsteps, unsigned epoch0, uint4 *pub, i
         const int n = gridDim.x * gridDim.y == 1 ? left : min(left, T);
         left -= n;
         for (int t = 0; t < n; ++t) {
-            // Branch-free, so that a thread's cells overlap: cells outside the
-            // inner region compute on whatever lies there and keep their value.
-            // Momentum predictor of the east and north faces of each cell
+            // Cells outside the inner region compute on whatever lies there and
+            // keep their value.  Momentum predictor and flux of the east and
+            // north faces of each cell
 #pragma unroll
             for (int k = 0; k < PER; ++k) {
                 const int q = tid + k * SWC_THREADS;
-                const bool wc = hh[q] > hmin;
-                const float ue = sw_face_mask(sw_predict(ru[k], p.gdt_dx, e[q + 1], re[k]), wc, hh[q + 1] > hmin);
-                const float vn = sw_face_mask(sw_predict(rv[k], p.gdt_dy, e[q + LW], re[k]), wc, hh[q + LW] > hmin);
-                ru[k] = m[k] & F_EAST ? ue : 0.0f;
-                rv[k] = m[k] & F_NORTH ? vn : 0.0f;
-                uu[q] = ru[k];
-                vv[q] = rv[k];
+                const float h = __fadd_rn(rH[k], re[k]), he = hh[q + 1], hn = hh[q + LW];
+                const bool wc = h > hmin, east = m[k] & F_EAST, north = m[k] & F_NORTH;
+                float a, b;
+                ru[k] = swc_face(sw_predict(ru[k], p.gdt_dx, e[q + 1], re[k]), wc && east, he > hmin && east, &a, &b);
+                const float f = __fmaf_rn(a, h, __fmul_rn(b, he));
+                rv[k] = swc_face(sw_predict(rv[k], p.gdt_dy, e[q + LW], re[k]), wc && north, hn > hmin && north, &a, &b);
+                const float g = __fmaf_rn(a, h, __fmul_rn(b, hn));
+                ff[q] = f;
+                gg[q] = g;
+                if (FREG) {
+                    rf[FREG ? k : 0] = f;
+                    rg[FREG ? k : 0] = g;
+                }
             }
             __syncthreads();
-            // continuity with upwind face fluxes; the masked eta* and the wet neighbours' count
+            // continuity; the masked eta* and the mask
 #pragma unroll
             for (int k = 0; k < PER; ++k) {
                 const int q = tid + k * SWC_THREADS;
-                const float h1 = hh[q], he = hh[q + 1], hw = hh[q - 1], hn = hh[q + LW], hs = hh[q - LW];
-                const float fe = sw_upwind(ru[k], h1, he);
-                const float fw = sw_upwind(uu[q - 1], hw, h1);
-                const float gn = sw_upwind(rv[k], h1, hn);
-                const float gs = sw_upwind(vv[q - LW], hs, h1);
-                const float es = __fsub_rn(re[k], __fmaf_rn(p.dt_dx, __fsub_rn(fe, fw), __fmul_rn(p.dt_dy, __fsub_rn(gn, gs))));
-                if constexpr (COEF) {
-                    const float cnt = ((he > hmin ? 1.0f : 0.0f) + (hw > hmin ? 1.0f : 0.0f)) +
-                                      ((hn > hmin ? 1.0f : 0.0f) + (hs > hmin ? 1.0f : 0.0f));
-                    rc[k] = __fsub_rn(1.0f, __fmul_rn(p.q, cnt));
-                } else {
-                    m[k] = (m[k] & 0xffu) + (he > hmin ? 0x100u : 0u) + (hw > hmin ? 0x100u : 0u) +
-                           (hn > hmin ? 0x100u : 0u) + (hs > hmin ? 0x100u : 0u);
-                }
+                const bool wc = __fadd_rn(rH[k], re[k]) > hmin;
+                const float f = FREG ? rf[FREG ? k : 0] : ff[q], g = FREG ? rg[FREG ? k : 0] : gg[q];
+                const float es = __fsub_rn(re[k], __fmaf_rn(p.dt_dx, __fsub_rn(f, ff[q - 1]),
+                                                            __fmul_rn(p.dt_dy, __fsub_rn(g, gg[q - LW]))));
                 re[k] = m[k] & F_INNER ? es : re[k];
-                we[q] = h1 > hmin ? re[k] : 0.0f;
+                we[q] = make_float2(wc ? re[k] : 0.0f, wc ? 1.0f : 0.0f);
+                m[k] = (m[k] & ~F_WET) | (wc ? F_WET : 0u);
             }
             __syncthreads();
             // masked Shapiro filter on wet cells; the next step's depth
 #pragma unroll
             for (int k = 0; k < PER; ++k) {
                 const int q = tid + k * SWC_THREADS;
-                const float sum = __fadd_rn(__fadd_rn(we[q + 1], we[q - 1]), __fadd_rn(we[q + LW], we[q - LW]));
-                const float c = COEF ? rc[COEF ? k : 0] : __fsub_rn(1.0f, __fmul_rn(p.q, (float)(m[k] >> 8)));
-                const float out = __fmaf_rn(p.q, sum, __fmul_rn(c, re[k]));
-                re[k] = (m[k] & F_INNER) && hh[q] > hmin ? out : re[k];
+                const float2 ae = we[q + 1], aw = we[q - 1], an = we[q + LW], as = we[q - LW];
+                const float sum = __fadd_rn(__fadd_rn(ae.x, aw.x), __fadd_rn(an.x, as.x));
+                const float cnt = (ae.y + aw.y) + (an.y + as.y);  // small integers: exact
+                const float out = __fmaf_rn(p.q, sum, __fmul_rn(__fsub_rn(1.0f, __fmul_rn(p.q, cnt)), re[k]));
+                re[k] = (m[k] & (F_INNER | F_WET)) == (F_INNER | F_WET) ? out : re[k];
                 e[q] = re[k];
                 hh[q] = __fadd_rn(rH[k], re[k]);
             }
