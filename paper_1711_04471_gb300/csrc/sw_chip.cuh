@@ -61,17 +61,6 @@ __device__ __forceinline__ void swc_store(uint4 *p, float a, float b, float c, u
                  ::"l"(p), "l"(lo), "l"(hi) : "memory");
 }
 
-// Velocity of a face and its parts that carry flux: vel as predicted, the
-// cells behind and ahead wet (both false: a wall).  The masked velocity's
-// positive part needs the cell behind to be wet, its negative part the cell
-// ahead (the rule of sw_face_mask).
-__device__ __forceinline__ float swc_face(float vel, bool wet_b, bool wet_a, float *pos, float *neg)
-{
-    *pos = wet_b ? fmaxf(vel, 0.0f) : 0.0f;
-    *neg = wet_a ? fminf(vel, 0.0f) : 0.0f;
-    return wet_b && wet_a ? vel : __fadd_rn(*pos, *neg);
-}
-
 // nsteps steps from (eta_in, u_in, v_in) to (eta_out, u_out, v_out).  pub:
 // two arrays of ny x nx words (NULL with a single tile); epoch0: number of
 // the last exchange of earlier launches.  Cooperative launch: grid (cx, cy),
@@ -147,9 +136,9 @@ sw_chip_kernel(SWDev p, SWChipPlan P, int nsteps, unsigned epoch0, uint4 *pub, i
                 const float h = __fadd_rn(rH[k], re[k]), he = hh[q + 1], hn = hh[q + LW];
                 const bool wc = h > hmin, east = m[k] & F_EAST, north = m[k] & F_NORTH;
                 float a, b;
-                ru[k] = swc_face(sw_predict(ru[k], p.gdt_dx, e[q + 1], re[k]), wc && east, he > hmin && east, &a, &b);
+                ru[k] = sw_face(sw_predict(ru[k], p.gdt_dx, e[q + 1], re[k]), wc && east, he > hmin && east, &a, &b);
                 const float f = __fmaf_rn(a, h, __fmul_rn(b, he));
-                rv[k] = swc_face(sw_predict(rv[k], p.gdt_dy, e[q + LW], re[k]), wc && north, hn > hmin && north, &a, &b);
+                rv[k] = sw_face(sw_predict(rv[k], p.gdt_dy, e[q + LW], re[k]), wc && north, hn > hmin && north, &a, &b);
                 const float g = __fmaf_rn(a, h, __fmul_rn(b, hn));
                 ff[q] = f;
                 gg[q] = g;

@@ -39,6 +39,17 @@ __device__ __forceinline__ float sw_face_mask(float vel, bool wet_behind, bool w
     return keep ? vel : 0.0f;
 }
 
+// Velocity of a face and its parts that carry flux: vel as predicted, the
+// cells behind and ahead wet (both false: a wall).  The masked velocity's
+// positive part needs the cell behind to be wet, its negative part the cell
+// ahead (the rule of sw_face_mask).
+__device__ __forceinline__ float sw_face(float vel, bool wet_b, bool wet_a, float *pos, float *neg)
+{
+    *pos = wet_b ? fmaxf(vel, 0.0f) : 0.0f;
+    *neg = wet_a ? fminf(vel, 0.0f) : 0.0f;
+    return wet_b && wet_a ? vel : __fadd_rn(*pos, *neg);
+}
+
 // The step's arithmetic is written with explicit round-to-nearest
 // intrinsics (no compiler-chosen multiply-add contraction), so the result
 // of a cell does not depend on the fusion depth or the tiling.

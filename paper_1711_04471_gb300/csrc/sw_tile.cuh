@@ -5,21 +5,23 @@
 // launch picks another height, so that the CTAs spread evenly over the
 // SMs) plus a halo of 2T cells on every side (the dependency radius of one
 // step is 2 cells) into shared memory, advances the whole tile T steps
-// there, and writes back the middle SWT_W x th cells.  Each step is three barrier-separated
-// phases over the tile: momentum predictor u', v'; continuity eta*;
-// masked Shapiro filter, which also forms the next step's depth h (in the
-// other of two h buffers, since this phase still reads the current one).
-// A thread keeps its own cells' values in registers (H never leaves
-// them); shared memory holds only what the neighbours read.  Cells past a
-// tile edge are not read (the results there are discarded halo); cells
-// outside the grid are loaded as H = eta = u = v = 0 and stay so, exactly
-// as in the streaming kernel.  Every operation is the streaming kernel's,
-// rounded in the same order (explicit round-to-nearest intrinsics), so the
-// two kernels give bitwise the same state.
+// there, and writes back the middle SWT_W x th cells.  Each step is three
+// barrier-separated phases over the tile: momentum predictor and face fluxes;
+// continuity eta*, stored multiplied by the wet mask and beside it; masked
+// Shapiro filter, which also forms the next step's depth.  A thread keeps
+// its own cells' values in registers (H never leaves them); shared memory
+// holds only what the neighbours read.  Cells past a tile edge hold discarded
+// halo; cells outside the grid are loaded as H = eta = u = v = 0 and stay so,
+// exactly as in the streaming kernel.  Every operation is the streaming
+// kernel's, rounded in the same order (explicit round-to-nearest
+// intrinsics), so the two kernels give bitwise the same state.
 //
 // Compared with the streaming kernel, a launch has no row-by-row pipeline:
 // its latency is one load, 3T short phases and one store, which is what
-// the small grids of the paper (500^2 .. 2000^2, a few MB) need.
+// the small grids of the paper (500^2 .. 2000^2, a few MB) need.  The phases
+// are bound by issued instructions: forming each face's flux once, instead of
+// on both sides of it, took the step from 9.63 to 8.75 us at 1100x1020 and
+// from 15.4 to 14.0 us at 1237x1501 (T = 2, balanced heights).
 #pragma once
 
 #include "sw_kernels.cuh"
@@ -30,7 +32,7 @@ constexpr int SWT_W = 32;           // written columns of a tile
 constexpr int SWT_H = 32;           // written rows of a tile unless the launch asks for another height
 constexpr int SWT_THREADS = 1024;   // about two cells per thread and phase: the phases are short, latency-bound loops
 constexpr int SWT_PER = 2;          // cells per thread
-constexpr int SWT_NC_MAX = SWT_PER * SWT_THREADS;  // cells of a tile with its halo: 6 arrays of them fill the 48 KB static limit
+constexpr int SWT_NC_MAX = SWT_PER * SWT_THREADS;  // cells of a tile with its halo: 6 words for each fill the 48 KB static limit
 constexpr int SWT_MAX_T = 3;        // a 32 x 32 tile with its halo fits up to T = 3
 
 // Most written rows of a tile of depth T: (SWT_W + 4T)(rows + 4T) <= SWT_NC_MAX
@@ -73,9 +75,17 @@ sw_tile_kernel(SWDev p, int th, const float *__restrict__ H, const float *__rest
     constexpr int LW = SWT_W + 2 * HALO;  // the row stride of the shared arrays stays a constant
     constexpr int PER = SWT_PER;
     const int LH = th + 2 * HALO, NC = LW * LH;  // NC <= SWT_NC_MAX
-    // neighbours' values only: each thread keeps its own cells' values in registers
-    __shared__ float e[SWT_NC_MAX], uu[SWT_NC_MAX], vv[SWT_NC_MAX], hh2[2][SWT_NC_MAX],
-        es[SWT_NC_MAX];  // depth double-buffered by step
+    // neighbours' values only: each thread keeps its own cells' values in
+    // registers.  Depth, elevation, fluxes through the east and north faces,
+    // masked eta* and wet mask.  Reads past an array's last row fall into the
+    // next one and are not used.
+    struct Shared {
+        float hh[SWT_NC_MAX], e[SWT_NC_MAX], ff[SWT_NC_MAX], gg[SWT_NC_MAX];
+        float2 we[SWT_NC_MAX];
+    };
+    __shared__ Shared sm;
+    float *const hh = sm.hh, *const e = sm.e, *const ff = sm.ff, *const gg = sm.gg;
+    float2 *const we = sm.we;
     const int x0 = blockIdx.x * SWT_W - HALO, y0 = blockIdx.y * th - HALO;
     const float hmin = p.hmin;
 
@@ -91,8 +101,9 @@ sw_tile_kernel(SWDev p, int th, const float *__restrict__ H, const float *__rest
     constexpr unsigned F_STORE = 1u << 12;  // written back (inside the written block and the grid)
     constexpr unsigned F_LOAD = 1u << 13;   // inside the grid: loaded (else H = eta = u = v = 0)
     constexpr unsigned F_CELL = 1u << 14;   // a cell of the tile (q < NC)
+    constexpr unsigned F_WET = 1u << 15;    // wet at the start of the step
     constexpr unsigned long long ROWS = swt_row_bits(T);
-    float re[PER], ru[PER], rv[PER], rH[PER], rh[PER], rs[PER];
+    float re[PER], ru[PER], rv[PER], rH[PER];
     unsigned m[PER];
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
@@ -136,81 +147,58 @@ sw_tile_kernel(SWDev p, int th, const float *__restrict__ H, const float *__rest
         re[k] = a;
         ru[k] = b;
         rv[k] = c;
-        rs[k] = 0.0f;
-        // depth of the first step, and the fields the neighbours read
-        rh[k] = __fadd_rn(rH[k], re[k]);
+        // the fields the neighbours read
         if (m[k] & F_CELL) {
-            hh2[0][q] = rh[k];
+            hh[q] = __fadd_rn(rH[k], re[k]);
             e[q] = re[k];
         }
     }
     __syncthreads();
-    // The step loop is unrolled so that each step's pair of h buffers is
-    // fixed at compile time.  The rolled loop (buffer picked from t at run
-    // time) gave states that differed from the streaming kernel at T = 3 in
-    // the bitwise tiling tests; the cause was not found, and the unrolled
-    // form matches bit for bit.
 #pragma unroll
     for (int t = 0; t < T; ++t) {
-        const float *hh = hh2[t & 1];
         const unsigned F_B = 1u << (3 * t), F_C = 1u << (3 * t + 1), F_D = 1u << (3 * t + 2);
-        // momentum predictor of the east and north faces of each cell
+        // momentum predictor and flux of the east and north faces of each cell
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
             if (!(m[k] & F_B)) continue;
             const int q = threadIdx.x + k * SWT_THREADS;
-            const bool wc = rh[k] > hmin;
-            float un = 0.0f, vn = 0.0f;
-            if (m[k] & F_EAST)
-                un = sw_face_mask(sw_predict(ru[k], p.gdt_dx, e[q + 1], re[k]), wc, hh[q + 1] > hmin);
-            if (m[k] & F_NORTH)
-                vn = sw_face_mask(sw_predict(rv[k], p.gdt_dy, e[q + LW], re[k]), wc, hh[q + LW] > hmin);
-            ru[k] = un;
-            rv[k] = vn;
-            uu[q] = un;
-            vv[q] = vn;
+            const float h = __fadd_rn(rH[k], re[k]), he = hh[q + 1], hn = hh[q + LW];
+            const bool wc = h > hmin, east = m[k] & F_EAST, north = m[k] & F_NORTH;
+            float a, b;
+            ru[k] = sw_face(sw_predict(ru[k], p.gdt_dx, e[q + 1], re[k]), wc && east, he > hmin && east, &a, &b);
+            ff[q] = __fmaf_rn(a, h, __fmul_rn(b, he));
+            rv[k] = sw_face(sw_predict(rv[k], p.gdt_dy, e[q + LW], re[k]), wc && north, hn > hmin && north, &a, &b);
+            gg[q] = __fmaf_rn(a, h, __fmul_rn(b, hn));
         }
         __syncthreads();
-        // continuity with upwind face fluxes
+        // continuity; the masked eta* and the mask
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
             if (!(m[k] & F_C)) continue;
             const int q = threadIdx.x + k * SWT_THREADS;
-            float out = re[k];
-            if (m[k] & F_INNER) {
-                const float h1 = rh[k];
-                const float fe = sw_upwind(ru[k], h1, hh[q + 1]);
-                const float fw = sw_upwind(uu[q - 1], hh[q - 1], h1);
-                const float gn = sw_upwind(rv[k], h1, hh[q + LW]);
-                const float gs = sw_upwind(vv[q - LW], hh[q - LW], h1);
-                out = __fsub_rn(re[k], __fmaf_rn(p.dt_dx, __fsub_rn(fe, fw), __fmul_rn(p.dt_dy, __fsub_rn(gn, gs))));
-            }
-            rs[k] = out;
-            es[q] = out;
+            const bool wc = __fadd_rn(rH[k], re[k]) > hmin, inner = m[k] & F_INNER;
+            const float fw = ff[inner ? q - 1 : q], gs = gg[inner ? q - LW : q];
+            const float es = __fsub_rn(re[k], __fmaf_rn(p.dt_dx, __fsub_rn(ff[q], fw),
+                                                        __fmul_rn(p.dt_dy, __fsub_rn(gg[q], gs))));
+            re[k] = inner ? es : re[k];
+            we[q] = make_float2(wc ? re[k] : 0.0f, wc ? 1.0f : 0.0f);
+            m[k] = (m[k] & ~F_WET) | (wc ? F_WET : 0u);
         }
         __syncthreads();
-        // masked Shapiro filter on wet cells
+        // masked Shapiro filter on wet cells; the next step's depth
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
             if (!(m[k] & F_D)) continue;
             const int q = threadIdx.x + k * SWT_THREADS;
-            float out = rs[k];
-            if ((m[k] & F_INNER) && rh[k] > hmin) {
-                const float we = hh[q + 1] > hmin ? 1.0f : 0.0f;
-                const float ww = hh[q - 1] > hmin ? 1.0f : 0.0f;
-                const float wn = hh[q + LW] > hmin ? 1.0f : 0.0f;
-                const float ws = hh[q - LW] > hmin ? 1.0f : 0.0f;
-                const float cnt = (we + ww) + (wn + ws);  // small integers: exact
-                const float sum = __fadd_rn(__fadd_rn(__fmul_rn(we, es[q + 1]), __fmul_rn(ww, es[q - 1])),
-                                            __fadd_rn(__fmul_rn(wn, es[q + LW]), __fmul_rn(ws, es[q - LW])));
-                out = __fmaf_rn(p.q, sum, __fmul_rn(__fsub_rn(1.0f, __fmul_rn(p.q, cnt)), rs[k]));
+            if ((m[k] & (F_INNER | F_WET)) == (F_INNER | F_WET)) {
+                const float2 ae = we[q + 1], aw = we[q - 1], an = we[q + LW], as = we[q - LW];
+                const float sum = __fadd_rn(__fadd_rn(ae.x, aw.x), __fadd_rn(an.x, as.x));
+                const float cnt = (ae.y + aw.y) + (an.y + as.y);  // small integers: exact
+                re[k] = __fmaf_rn(p.q, sum, __fmul_rn(__fsub_rn(1.0f, __fmul_rn(p.q, cnt)), re[k]));
             }
-            re[k] = out;
             if (t + 1 < T) {
-                // the next step's depth goes to the other buffer: this phase still reads hh
-                rh[k] = __fadd_rn(rH[k], out);
-                hh2[(t + 1) & 1][q] = rh[k];
-                e[q] = out;
+                hh[q] = __fadd_rn(rH[k], re[k]);
+                e[q] = re[k];
             }
         }
         if (t + 1 < T) __syncthreads();
