@@ -157,7 +157,8 @@ sw_chip_kernel(SWDev p, SWChipPlan P, int nsteps, unsigned epoch0, uint4 *pub, i
                 const float es = __fsub_rn(re[k], __fmaf_rn(p.dt_dx, __fsub_rn(f, ff[q - 1]),
                                                             __fmul_rn(p.dt_dy, __fsub_rn(g, gg[q - LW]))));
                 re[k] = m[k] & F_INNER ? es : re[k];
-                we[q] = make_float2(wc ? re[k] : 0.0f, wc ? 1.0f : 0.0f);
+                const float w = wc ? 1.0f : 0.0f;
+                we[q] = make_float2(__fmul_rn(w, re[k]), w);
                 m[k] = (m[k] & ~F_WET) | (wc ? F_WET : 0u);
             }
             __syncthreads();

@@ -31,33 +31,23 @@ constexpr int SW_NOALLOC_MAX_SIDE = 1 << 20;  // largest nx, ny accepted by sw_v
 // translation unit that includes this header).
 static __device__ unsigned g_sw_bounds;
 
-// Wet/dry face rule: keep the predicted velocity if both cells are wet, or
-// if it flows out of a wet cell; otherwise the face is closed.
-__device__ __forceinline__ float sw_face_mask(float vel, bool wet_behind, bool wet_ahead)
-{
-    const bool keep = (wet_behind && wet_ahead) || (wet_behind && vel > 0.0f) || (wet_ahead && vel < 0.0f);
-    return keep ? vel : 0.0f;
-}
-
-// Velocity of a face and its parts that carry flux: vel as predicted, the
-// cells behind and ahead wet (both false: a wall).  The masked velocity's
-// positive part needs the cell behind to be wet, its negative part the cell
-// ahead (the rule of sw_face_mask).
+// Wet/dry face rule: the velocity `vel` predicted on a face between a cell
+// behind it and a cell ahead stays if both cells are wet or if it flows out
+// of a wet cell; otherwise the face is closed (and so is a wall: both flags
+// false).  pos and neg are the parts of the result that carry water out of
+// the cell behind and out of the cell ahead.
 __device__ __forceinline__ float sw_face(float vel, bool wet_b, bool wet_a, float *pos, float *neg)
 {
     *pos = wet_b ? fmaxf(vel, 0.0f) : 0.0f;
     *neg = wet_a ? fminf(vel, 0.0f) : 0.0f;
-    return wet_b && wet_a ? vel : __fadd_rn(*pos, *neg);
+    return wet_b & wet_a ? vel : __fadd_rn(*pos, *neg);
 }
 
 // The step's arithmetic is written with explicit round-to-nearest
 // intrinsics (no compiler-chosen multiply-add contraction), so the result
-// of a cell does not depend on the fusion depth or the tiling.
-__device__ __forceinline__ float sw_upwind(float vel, float h_behind, float h_ahead)
-{
-    return __fmaf_rn(fmaxf(vel, 0.0f), h_behind, __fmul_rn(fminf(vel, 0.0f), h_ahead));
-}
-
+// of a cell does not depend on the fusion depth or the tiling.  A face's
+// upwind flux is fma(pos, h behind, neg x h ahead).
+//
 // u - c (e_ahead - e_behind): the momentum predictor of one face.
 __device__ __forceinline__ float sw_predict(float vel, float c, float e_ahead, float e_behind)
 {

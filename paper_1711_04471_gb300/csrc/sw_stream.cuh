@@ -8,20 +8,30 @@
 // one row per iteration.  Time level t -> t+1 is a pipeline stage: stage t
 // receives a row of level t and emits the level-(t+1) row two rows below
 // it (the y-radius of one step's dependency cone).  Stage t+1 consumes
-// what stage t emitted in the previous iteration, so all stages share the
-// three block barriers of an iteration; stage t works 3t rows behind
-// stage 0 and the strip's output row trails the input row by 3T-1.
+// what stage t emitted in the previous iteration; stage t works 3t rows
+// behind stage 0 and the strip's output row trails the input row by 3T-1.
 //
 // Each thread keeps the y-neighbours of its own column in registers (the
 // rolling window below); x-neighbours go through per-stage shared-memory
 // line buffers.  Global memory is touched once per fused launch: level 0
-// rows (eta, u, v, H) are loaded two rows ahead, level T rows are stored.
+// rows (eta, u, v, H) are loaded four rows ahead, level T rows are stored.
 //
-// One step on row n (level t -> t+1), with h = H + eta, wet = h > hmin:
-//   u'(n)    = mask(u - g dt/dx (eta_e - eta_c))       (needs eta(x+1, n))
-//   v'(n-1)  = mask(v - g dt/dy (eta(n) - eta(n-1)))
-//   eta*(n-1)= eta - dt/dx (F_e - F_w) - dt/dy (G_n - G_s), upwind fluxes
-//   eta+(n-2)= masked Shapiro filter of eta* (needs eta*(n-3..n-1))
+// One step on row n (level t -> t+1), with h = H + eta, w = h > hmin:
+//   u'(n), F(n)     = face(u - g dt/dx (eta_e - eta_c))   (needs eta, h at (x+1, n))
+//   v'(n-1), G(n-1) = face(v - g dt/dy (eta(n) - eta(n-1)))
+//   eta*(n-1) = eta - dt/dx (F - F_w) - dt/dy (G - G_s)   (F_w(n-1): the line of the last iteration)
+//   eta+(n-2) = Shapiro filter of w eta*                  (the lines' row n-2: the last iteration's)
+// Only (eta, h) are read in the iteration that publishes them, so one
+// barrier per row is enough: a line slot is rewritten two iterations after
+// it was filled, with a barrier between its last read and the rewrite.
+//
+// Bound by issued instructions (86 per cell and step, 58 % of the issue
+// slots) and the latencies that four warps per scheduler leave open.  Each
+// face's flux is formed once, w eta* travels with w, loads and stores are
+// predicated, a wall is a wet threshold of infinity.  With three barriers
+// per row, branches and the fluxes formed on both sides of every face a step
+// took (T = 3) at 4096x4096 75 us, now 57; 2000x2000 23.5, 17.0; 1237x1501
+// 15.2, 9.5.
 #pragma once
 
 #include <type_traits>
@@ -36,13 +46,13 @@ constexpr int SWS_LINE = SWS_THREADS + 2 * SWS_PAD;
 
 // Rolling per-stage window of one column (registers).
 struct SWStageRegs {
-    float eta1, eta2;   // eta at rows n-1, n-2 (level t)
-    float h1, h2, h3;   // h at rows n-1, n-2, n-3
-    float H1, H2;       // still-water depth at rows n-1, n-2
-    float v1;           // v (level t) at row n-1
-    float vp2;          // v' at row n-2
-    float up1, up2;     // u' at rows n-1, n-2
-    float es2, es3;     // eta* at rows n-2, n-3
+    float eta1, h1, v1;  // level-t row n-1
+    float H1, H2;        // still-water depth at rows n-1, n-2
+    float F1, G2;        // fluxes: F at row n-1, G at row n-2
+    float up1, up2, vp2; // u' at rows n-1, n-2, v' at row n-2
+    float es2;           // eta* at row n-2
+    float we2, we3;      // w eta* at rows n-2, n-3
+    float w1, w2, w3;    // w at rows n-1, n-2, n-3
 };
 
 // A row of one column handed from a stage to the next (or loaded / stored).
@@ -52,10 +62,9 @@ struct SWRow {
 
 // Per-stage shared line buffers.
 struct SWStageLines {
-    float eta[2][SWS_LINE];
-    float h[4][SWS_LINE];
-    float up[2][SWS_LINE];
-    float es[2][SWS_LINE];
+    float2 eh[2][SWS_LINE];  // eta, h of the incoming row
+    float2 ws[2][SWS_LINE];  // w eta*, w
+    float F[2][SWS_LINE];    // flux through the east faces
 };
 
 // Loads of the level-0 rows: through the read-only path when the inputs
@@ -64,11 +73,24 @@ struct SWStageLines {
 // CTAs rewrite the buffers between levels.
 enum class SWLoad { ReadOnly, L2 };
 
+// *ptr if ok, else 0; and *ptr = v if ok: one predicated access, no branch.
 template <SWLoad LP>
-__device__ __forceinline__ float sw_load(const float *ptr)
+__device__ __forceinline__ float sw_load(const float *ptr, bool ok)
 {
-    if constexpr (LP == SWLoad::ReadOnly) return __ldg(ptr);
-    else return __ldcg(ptr);
+    float v;
+    if constexpr (LP == SWLoad::ReadOnly)
+        asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n mov.f32 %0, 0f00000000;\n @p ld.global.nc.f32 %0, [%1];\n}"
+                     : "=f"(v) : "l"(ptr), "r"((unsigned)ok));
+    else
+        asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n mov.f32 %0, 0f00000000;\n @p ld.global.cg.f32 %0, [%1];\n}"
+                     : "=f"(v) : "l"(ptr), "r"((unsigned)ok) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void sw_store(float *ptr, float v, bool ok)
+{
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p st.global.f32 [%0], %1;\n}"
+                 :: "l"(ptr), "f"(v), "r"((unsigned)ok) : "memory");
 }
 
 // One (strip, row segment) work item: T fused steps of the columns of
@@ -95,143 +117,123 @@ __device__ __forceinline__ void sw_stream_tile(const SWDev &p, int strip, int r0
         const int st = x >> 1;
         const int side = (x & 1) ? SWS_LINE - 1 : 0;
         for (int k = 0; k < 2; ++k) {
-            lines[st].eta[k][side] = 0.0f;
-            lines[st].up[k][side] = 0.0f;
-            lines[st].es[k][side] = 0.0f;
+            lines[st].eh[k][side] = lines[st].ws[k][side] = make_float2(0.0f, 0.0f);
+            lines[st].F[k][side] = 0.0f;
         }
-        for (int k = 0; k < 4; ++k) lines[st].h[k][side] = 0.0f;
     }
 
-    const float hmin = p.hmin;
+    const float hmin = p.hmin, inf = __int_as_float(0x7f800000);
+    const float hmin_u = u_open ? hmin : inf;  // wet threshold of the east face: nothing is above it at a wall
     SWStageRegs R[T];
     SWRow mail[T];  // mail[t]: level-(t+1) row emitted by stage t last iteration
 #pragma unroll
     for (int t = 0; t < T; ++t) {
-        R[t] = SWStageRegs{0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+        R[t] = SWStageRegs{};
         mail[t] = SWRow{0, 0, 0, 0};
     }
 
     const long long extent = (long long)p.ny * p.pitch;  // elements of each field of this grid
     auto load_row = [&](int n) {
-        SWRow r{0.0f, 0.0f, 0.0f, 0.0f};
-        if (col_in && n >= 0 && n < p.ny && GBSW_INBOUNDS((long long)n * p.pitch + gi, extent, &g_sw_bounds)) {
-            const size_t g = (size_t)n * p.pitch + gi;
-            r.eta = sw_load<LP>(eta_in + g);
-            r.u = sw_load<LP>(u_in + g);
-            r.v = sw_load<LP>(v_in + g);
-            r.H = sw_load<LP>(H + g);
-        }
+        const long long g = (long long)n * p.pitch + gi;
+        const bool ok = col_in & ((unsigned)n < (unsigned)p.ny) && GBSW_INBOUNDS(g, extent, &g_sw_bounds);
+        SWRow r;
+        r.eta = sw_load<LP>(eta_in + g, ok);
+        r.u = sw_load<LP>(u_in + g, ok);
+        r.v = sw_load<LP>(v_in + g, ok);
+        r.H = sw_load<LP>(H + g, ok);
         return r;
     };
 
-    // The ring slots of the line buffers repeat every 4 rows; the row loop
-    // is unrolled by 4 so every slot index and the register window shift
-    // are resolved at compile time.
+    // The row loop is unrolled by 4 so that every line slot and the shift of
+    // the register window are resolved at compile time.
     const int n_first = (r0 - 2 * T) & ~3;    // first level-0 row that matters, rounded down
     const int n_last = r1 - 1 + 3 * T - 1;    // iteration that emits output row r1-1
-    SWRow pre0 = load_row(n_first), pre1 = load_row(n_first + 1);
+    SWRow pre[4];  // the rows ahead: four cover the latency of a load from DRAM
+#pragma unroll
+    for (int k = 0; k < 4; ++k) pre[k] = load_row(n_first + k);
 
     auto iteration = [&](auto phase, int n4) {
         constexpr int P = decltype(phase)::value;  // n & 3
         const int n = n4 + P;
         SWRow in[T];
-        in[0] = pre0;
-        pre0 = pre1;
-        pre1 = load_row(n + 2);
+        in[0] = pre[P];
+        pre[P] = load_row(n + 4);
 #pragma unroll
         for (int t = 1; t < T; ++t) in[t] = mail[t - 1];
 
-        // phase 1: publish eta and h of the incoming row of every stage
+        // publish eta and h of the incoming row of every stage
         float hn[T];
 #pragma unroll
         for (int t = 0; t < T; ++t) {
-            const int s0 = (P - 3 * t) & 3;  // slot of row m = n - 3t
+            const int s0 = (P - 3 * t) & 1;  // slot of row m = n - 3t
             hn[t] = __fadd_rn(in[t].H, in[t].eta);
-            lines[t].eta[s0 & 1][c] = in[t].eta;
-            lines[t].h[s0][c] = hn[t];
+            lines[t].eh[s0][c] = make_float2(in[t].eta, hn[t]);
         }
         __syncthreads();
-        // phase 2: momentum predictor u'(m), v'(m-1)
-        float un[T], vn1[T];
+        // what the neighbour columns published, of all stages at once: the
+        // stages' arithmetic interleaves between the loads and the stores
+        float2 ee[T], ae[T], aw[T];
+        float Fw[T], Fn[T], we[T];
 #pragma unroll
         for (int t = 0; t < T; ++t) {
-            const int s0 = (P - 3 * t) & 3;
+            const int s0 = (P - 3 * t) & 1, s1 = s0 ^ 1;  // slots of row m (and m-2), of row m-1
+            ee[t] = lines[t].eh[s0][c + 1];
+            Fw[t] = lines[t].F[s1][c - 1];
+            ae[t] = lines[t].ws[s0][c + 1];
+            aw[t] = lines[t].ws[s0][c - 1];
+        }
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
             const int m = n - 3 * t;
-            const bool wc = hn[t] > hmin;
-            float uv = 0.0f;
-            if (u_open) {
-                const float ee = lines[t].eta[s0 & 1][c + 1];
-                const bool we = lines[t].h[s0][c + 1] > hmin;
-                uv = sw_face_mask(sw_predict(in[t].u, p.gdt_dx, ee, in[t].eta), wc, we);
-            }
-            un[t] = uv;
-            float vv = 0.0f;
-            if (m - 1 >= 0 && m - 1 < p.ny - 1)
-                vv = sw_face_mask(sw_predict(R[t].v1, p.gdt_dy, in[t].eta, R[t].eta1), R[t].h1 > hmin, wc);
-            vn1[t] = vv;
-            lines[t].up[s0 & 1][c] = uv;
-        }
-        __syncthreads();
-        // phase 3: continuity eta*(m-1)
-        float es1[T];
-#pragma unroll
-        for (int t = 0; t < T; ++t) {
-            const int s1 = (P - 3 * t - 1) & 3;  // slot of row m-1
-            const float uw = lines[t].up[s1 & 1][c - 1];
-            const float he = lines[t].h[s1][c + 1], hw = lines[t].h[s1][c - 1];
-            const float h1 = R[t].h1;
-            const float fe = sw_upwind(R[t].up1, h1, he);
-            const float fw = sw_upwind(uw, hw, h1);
-            const float gn = sw_upwind(vn1[t], h1, hn[t]);
-            const float gs = sw_upwind(R[t].vp2, R[t].h2, h1);
-            es1[t] = __fsub_rn(R[t].eta1, __fmaf_rn(p.dt_dx, __fsub_rn(fe, fw), __fmul_rn(p.dt_dy, __fsub_rn(gn, gs))));
-            lines[t].es[s1 & 1][c] = es1[t];
-        }
-        __syncthreads();
-        // phase 4: Shapiro filter eta+(m-2), emit the level-(t+1) row m-2
-#pragma unroll
-        for (int t = 0; t < T; ++t) {
-            const int s2 = (P - 3 * t - 2) & 3;  // slot of row m-2
-            const float es2 = R[t].es2;
-            float out = es2;
-            if (R[t].h2 > hmin) {
-                const float we = lines[t].h[s2][c + 1] > hmin ? 1.0f : 0.0f;
-                const float ww = lines[t].h[s2][c - 1] > hmin ? 1.0f : 0.0f;
-                const float wn = R[t].h1 > hmin ? 1.0f : 0.0f;
-                const float ws = R[t].h3 > hmin ? 1.0f : 0.0f;
-                const float ee = lines[t].es[s2 & 1][c + 1];
-                const float ew = lines[t].es[s2 & 1][c - 1];
-                const float cnt = (we + ww) + (wn + ws);  // small integers: exact
-                const float sum = __fadd_rn(__fadd_rn(__fmul_rn(we, ee), __fmul_rn(ww, ew)),
-                                            __fadd_rn(__fmul_rn(wn, es1[t]), __fmul_rn(ws, R[t].es3)));
-                out = __fmaf_rn(p.q, sum, __fmul_rn(__fsub_rn(1.0f, __fmul_rn(p.q, cnt)), es2));
-            }
-            mail[t] = SWRow{out, R[t].up2, R[t].vp2, R[t].H2};
-            // roll the window
             SWStageRegs &r = R[t];
-            r.eta2 = r.eta1;
+            float a, b;
+            // momentum predictor and fluxes: u'(m), F(m), v'(m-1), G(m-1)
+            const float un = sw_face(sw_predict(in[t].u, p.gdt_dx, ee[t].x, in[t].eta), hn[t] > hmin_u,
+                                     ee[t].y > hmin_u, &a, &b);
+            Fn[t] = __fmaf_rn(a, hn[t], __fmul_rn(b, ee[t].y));
+            const float hmin_v = (unsigned)(m - 1) < (unsigned)(p.ny - 1) ? hmin : inf;
+            const float vn = sw_face(sw_predict(r.v1, p.gdt_dy, in[t].eta, r.eta1), r.h1 > hmin_v,
+                                     hn[t] > hmin_v, &a, &b);
+            const float Gn = __fmaf_rn(a, r.h1, __fmul_rn(b, hn[t]));
+            // continuity: eta*(m-1)
+            const float es = __fsub_rn(r.eta1, __fmaf_rn(p.dt_dx, __fsub_rn(r.F1, Fw[t]), __fmul_rn(p.dt_dy, __fsub_rn(Gn, r.G2))));
+            we[t] = __fmul_rn(r.w1, es);
+            // Shapiro filter: eta+(m-2); emit the level-(t+1) row m-2
+            const float cnt = (ae[t].y + aw[t].y) + (r.w1 + r.w3);  // small integers: exact
+            const float sum = __fadd_rn(__fadd_rn(ae[t].x, aw[t].x), __fadd_rn(we[t], r.we3));
+            const float flt = __fmaf_rn(p.q, sum, __fmul_rn(__fsub_rn(1.0f, __fmul_rn(p.q, cnt)), r.es2));
+            mail[t] = SWRow{r.w2 != 0.0f ? flt : r.es2, r.up2, r.vp2, r.H2};
+            // roll the window
             r.eta1 = in[t].eta;
-            r.h3 = r.h2;
-            r.h2 = r.h1;
             r.h1 = hn[t];
+            r.v1 = in[t].v;
             r.H2 = r.H1;
             r.H1 = in[t].H;
-            r.v1 = in[t].v;
-            r.vp2 = vn1[t];
+            r.F1 = Fn[t];
+            r.G2 = Gn;
             r.up2 = r.up1;
-            r.up1 = un[t];
-            r.es3 = r.es2;
-            r.es2 = es1[t];
+            r.up1 = un;
+            r.vp2 = vn;
+            r.es2 = es;
+            r.we3 = r.we2;
+            r.we2 = we[t];
+            r.w3 = r.w2;
+            r.w2 = r.w1;
+            r.w1 = hn[t] > hmin ? 1.0f : 0.0f;
+        }
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            const int s0 = (P - 3 * t) & 1, s1 = s0 ^ 1;
+            lines[t].F[s0][c] = Fn[t];
+            lines[t].ws[s1][c] = make_float2(we[t], R[t].w2);
         }
         // the last stage's row is final: level T at row n - 3T + 1
         const int out_row = n - 3 * T + 1;
-        if (owned && out_row >= r0 && out_row < r1 &&
-            GBSW_INBOUNDS((long long)out_row * p.pitch + gi, extent, &g_sw_bounds)) {
-            const size_t g = (size_t)out_row * p.pitch + gi;
-            eta_out[g] = mail[T - 1].eta;
-            u_out[g] = mail[T - 1].u;
-            v_out[g] = mail[T - 1].v;
-        }
+        const long long g = (long long)out_row * p.pitch + gi;
+        const bool ok = owned & ((unsigned)(out_row - r0) < (unsigned)(r1 - r0)) && GBSW_INBOUNDS(g, extent, &g_sw_bounds);
+        sw_store(eta_out + g, mail[T - 1].eta, ok);
+        sw_store(u_out + g, mail[T - 1].u, ok);
+        sw_store(v_out + g, mail[T - 1].v, ok);
     };
 
 #pragma unroll 1

@@ -181,7 +181,8 @@ sw_tile_kernel(SWDev p, int th, const float *__restrict__ H, const float *__rest
             const float es = __fsub_rn(re[k], __fmaf_rn(p.dt_dx, __fsub_rn(ff[q], fw),
                                                         __fmul_rn(p.dt_dy, __fsub_rn(gg[q], gs))));
             re[k] = inner ? es : re[k];
-            we[q] = make_float2(wc ? re[k] : 0.0f, wc ? 1.0f : 0.0f);
+            const float w = wc ? 1.0f : 0.0f;
+            we[q] = make_float2(__fmul_rn(w, re[k]), w);
             m[k] = (m[k] & ~F_WET) | (wc ? F_WET : 0u);
         }
         __syncthreads();
