@@ -12,8 +12,9 @@
 // sw_batch_step captures the launch in a CUDA graph, so an nsteps call is
 // one graph launch however many instances there are.
 //
-// (T, rows per item) are chosen by sw_batch_autotune, which times the
-// candidates on the batch itself and can cache the choice in a text file.
+// (T, rows per item) are picked from the sizes (pick_rows) unless a tiling is
+// set, or by sw_batch_autotune, which times the candidates on the batch
+// itself and can cache the choice in a text file.
 #include <math.h>
 #include <stdio.h>
 #include <stdlib.h>
@@ -54,6 +55,7 @@ struct BatchDev {
 };
 
 constexpr long long SPIN_LIMIT = 20000000;  // ~ seconds; a level takes milliseconds
+constexpr int BATCH_T = 3;                  // depth of the automatic tiling
 constexpr int VOL_BLOCKS = 16;              // volume partial blocks per instance
 
 // Grid-wide barrier for a cooperative launch.  Returns false (in every
@@ -181,7 +183,9 @@ struct gbsw_sw_batch {
     int *status;
     double *partials, *area, *vol;
     int cur;
-    int T, rows;         // current tiling
+    int T, rows;         // tiling as set, tuned or reported
+    bool automatic;      // step with depth BATCH_T and pick_rows() instead
+    int auto_rows;       // pick_rows(), 0 until computed
     int grid_cache[8];   // co-resident CTAs per T
     std::map<long long, cudaGraphExec_t> graphs;  // key: nsteps * 2 + cur
 };
@@ -220,14 +224,57 @@ gbsw_status build_items(gbsw_sw_batch *b, int T, int rows)
 }
 
 template <int T>
-gbsw_status launch_batch(gbsw_sw_batch *b, cudaStream_t s, int nlevels, int cur0, unsigned *counters)
+gbsw_status batch_grid(gbsw_sw_batch *b)
 {
-    int &grid = b->grid_cache[T];
-    if (grid == 0) {
+    if (b->grid_cache[T] == 0) {
         int per_sm = 0;
         GBSW_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sw_batch_kernel<T>, SWS_THREADS, 0));
-        grid = std::max(1, per_sm) * sm_count();
+        b->grid_cache[T] = std::max(1, per_sm) * sm_count();
     }
+    return GBSW_OK;
+}
+
+// Rows of an item in the automatic tiling: those that make the shortest
+// level.  The co-resident CTAs take the items in ceil(items / CTAs) rounds,
+// each as long as the item's rows and its pipeline's fill (5T).  With 128
+// rows whatever the sizes, most CTAs of a small ensemble had no item: 12
+// grids of 66 .. 471 cells a side 28.0 us per step, now 7.8; 20 grids of
+// 67 .. 916 29.6, 25.3.
+gbsw_status pick_rows(gbsw_sw_batch *b, int *rows)
+{
+    if (b->auto_rows == 0) {
+        const gbsw_status st = batch_grid<BATCH_T>(b);
+        if (st != GBSW_OK) return st;
+        const long long ctas = b->grid_cache[BATCH_T];
+        long long best = -1;
+        for (int r = 128; r >= 8; r -= 8) {
+            long long n = 0;
+            for (const gbsw_sw_params &p : b->params)
+                n += (long long)ceil_div(p.nx, SWS_THREADS - 4 * BATCH_T) * ceil_div(p.ny, r);
+            const long long cost = (n + ctas - 1) / ctas * (r + 5 * BATCH_T);
+            if (best < 0 || cost < best) {
+                best = cost;
+                b->auto_rows = r;
+            }
+        }
+    }
+    *rows = b->auto_rows;
+    return GBSW_OK;
+}
+
+void set_automatic(gbsw_sw_batch *b)
+{
+    if (!b->automatic) free_graphs(b);
+    b->automatic = true;
+}
+
+int step_T(const gbsw_sw_batch *b) { return b->automatic ? BATCH_T : b->T; }
+
+template <int T>
+gbsw_status launch_batch(gbsw_sw_batch *b, cudaStream_t s, int nlevels, int cur0, unsigned *counters)
+{
+    const gbsw_status st = batch_grid<T>(b);
+    if (st != GBSW_OK) return st;
     BatchDev B;
     B.inst = b->inst;
     B.items = b->items[T];
@@ -244,7 +291,7 @@ gbsw_status launch_batch(gbsw_sw_batch *b, cudaStream_t s, int nlevels, int cur0
     B.status = b->status;
     B.spin_limit = fault_injected("sync_timeout") ? 0 : SPIN_LIMIT;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = dim3(b->grid_cache[T]);
     cfg.blockDim = dim3(SWS_THREADS);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = s;
@@ -273,10 +320,10 @@ gbsw_status launch_levels(gbsw_sw_batch *b, cudaStream_t s, int T, int nlevels, 
 // both depths must exist.
 gbsw_status enqueue_steps(gbsw_sw_batch *b, cudaStream_t s, int nsteps, int cur0)
 {
-    const int full = nsteps / b->T, tail = nsteps % b->T;
+    const int T = step_T(b), full = nsteps / T, tail = nsteps % T;
     GBSW_CUDA_TRY(cudaMemsetAsync(b->counters, 0, (size_t)(full + 1) * sizeof(unsigned), s));
     gbsw_status st = GBSW_OK;
-    if (full > 0) st = launch_levels(b, s, b->T, full, cur0, b->counters);
+    if (full > 0) st = launch_levels(b, s, T, full, cur0, b->counters);
     if (st == GBSW_OK && tail > 0) st = launch_levels(b, s, tail, 1, (cur0 + full) & 1, b->counters + full);
     return st;
 }
@@ -307,8 +354,9 @@ gbsw_status sw_batch_create(int n, const gbsw_sw_params *params, const double *c
     b->n = n;
     b->stream = (cudaStream_t)stream;
     b->params.assign(params, params + n);
-    b->T = 3;
+    b->T = BATCH_T;
     b->rows = 128;
+    b->automatic = true;
     long long off = 0;
     std::vector<double> area(n);
     for (int m = 0; m < n; ++m) {
@@ -394,7 +442,8 @@ gbsw_status sw_batch_set_tiling(gbsw_sw_batch *b, int steps_per_level, int rows_
 {
     if (!b || steps_per_level < 1 || steps_per_level > 4 || rows_per_item < 8 || rows_per_item > 65536)
         return GBSW_ERR_ARG;
-    if (b->T != steps_per_level || b->rows != rows_per_item) free_graphs(b);
+    if (b->T != steps_per_level || b->rows != rows_per_item || b->automatic) free_graphs(b);
+    b->automatic = false;
     b->T = steps_per_level;
     b->rows = rows_per_item;
     return GBSW_OK;
@@ -413,10 +462,12 @@ gbsw_status sw_batch_step(gbsw_sw_batch *b, int nsteps)
     gbsw::NvtxRange nvtx_range("sw_batch_step");
     if (!b || nsteps < 0) return GBSW_ERR_ARG;
     if (nsteps == 0) return GBSW_OK;
-    const int full = nsteps / b->T, tail = nsteps % b->T;
+    const int T = step_T(b), full = nsteps / T, tail = nsteps % T;
     gbsw_status st = ensure_levels(b, full + 1);
-    if (st == GBSW_OK) st = build_items(b, b->T, b->rows);
-    if (st == GBSW_OK && tail > 0) st = build_items(b, tail, b->rows);
+    int rows = b->rows;
+    if (st == GBSW_OK && b->automatic) st = pick_rows(b, &rows);
+    if (st == GBSW_OK) st = build_items(b, T, rows);
+    if (st == GBSW_OK && tail > 0) st = build_items(b, tail, rows);
     if (st != GBSW_OK) return st;
     const long long key = (long long)nsteps * 2 + b->cur;
     auto it = b->graphs.find(key);
@@ -540,8 +591,10 @@ gbsw_status sw_batch_get_state(gbsw_sw_batch *b, int m, float *eta, float *u, fl
     return GBSW_OK;
 }
 
-/* Time every (T, rows) candidate on the batch itself (state saved and
- * restored), keep the fastest.  cache_path may be NULL. */
+/* Time every (T, rows) candidate and the automatic tiling on the batch
+ * itself (state saved and restored), keep the fastest; the fastest pair is
+ * reported.  cache_path may be NULL; a line of the file is the key, the pair
+ * and "auto" if the automatic tiling is kept. */
 gbsw_status sw_batch_autotune(gbsw_sw_batch *b, int trial_steps, const char *cache_path, int *T_out, int *rows_out)
 {
     gbsw::NvtxRange nvtx_range("sw_batch_autotune");
@@ -570,11 +623,12 @@ gbsw_status sw_batch_autotune(gbsw_sw_batch *b, int trial_steps, const char *cac
         if (f) {
             char line[512];
             while (fgets(line, sizeof(line), f)) {
-                char k[400];
+                char k[400], mode[8] = "";
                 int T = 0, rows = 0;
-                if (sscanf(line, "%399s %d %d", k, &T, &rows) == 3 && strcmp(k, key) == 0) {
+                if (sscanf(line, "%399s %d %d %7s", k, &T, &rows, mode) >= 3 && strcmp(k, key) == 0) {
                     fclose(f);
                     gbsw_status st = sw_batch_set_tiling(b, T, rows);
+                    if (st == GBSW_OK && strcmp(mode, "auto") == 0) set_automatic(b);
                     if (T_out) *T_out = T;
                     if (rows_out) *rows_out = rows;
                     return st;
@@ -620,6 +674,20 @@ gbsw_status sw_batch_autotune(gbsw_sw_batch *b, int trial_steps, const char *cac
                 bestR = R;
             }
         }
+    // the automatic tiling
+    bool automatic = false;
+    if (st == GBSW_OK) {
+        set_automatic(b);
+        const int steps = std::max(BATCH_T, trial_steps / BATCH_T * BATCH_T);
+        if ((st = sw_batch_step(b, steps)) == GBSW_OK) {
+            cudaEventRecord(e0, b->stream);
+            st = sw_batch_step(b, steps);
+            cudaEventRecord(e1, b->stream);
+        }
+        float ms = 0.0f;
+        if (st == GBSW_OK && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess)
+            automatic = ms / (float)steps < best;
+    }
     // restore the state
     b->cur = c0;
     cudaMemcpyAsync(b->eta[c0], save[0], fb, cudaMemcpyDeviceToDevice, b->stream);
@@ -631,10 +699,11 @@ gbsw_status sw_batch_autotune(gbsw_sw_batch *b, int trial_steps, const char *cac
     cudaEventDestroy(e1);
     if (st != GBSW_OK) return st;
     st = sw_batch_set_tiling(b, bestT, bestR);
+    if (automatic) set_automatic(b);
     if (cache_path) {
         FILE *f = fopen(cache_path, "a");
         if (f) {
-            fprintf(f, "%s %d %d\n", key, bestT, bestR);
+            fprintf(f, automatic ? "%s %d %d auto\n" : "%s %d %d\n", key, bestT, bestR);
             fclose(f);
         }
     }
