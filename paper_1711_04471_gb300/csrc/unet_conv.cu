@@ -19,6 +19,35 @@ constexpr int CONV_THREADS = 128;
 
 __device__ __forceinline__ void set_status(int *status, int code) { atomicCAS(status, DEV_OK, code); }
 
+// Thread 0: the tile at (x0, y0, z0) shifted by (dx, dy, dz), NCG channel
+// groups, into slabs of 2048 bytes at dst (128 * NCG * 16 bytes arrive on bar).
+template <int NCG>
+__device__ __forceinline__ void load_tile(uint8_t *dst, const CUtensorMap *map, uint64_t *bar, const ConvGeom &g, int x0,
+                                          int y0, int z0, int dx, int dy, int dz)
+{
+    if (g.load == LOAD_SAMPLES) {
+        tc::tma_load_5d(dst, map, bar, 8 * dx, dy, z0 % g.D + dz, z0 / g.D, 0);
+        return;
+    }
+    const bool rows = g.load == LOAD_ROWS;
+    if (g.box_z == 1) {
+        const int z = z0 % g.D + dz, zsrc = z >= 0 && z < g.D ? z0 + dz : -1;
+        if (rows) tc::tma_load_5d(dst, map, bar, 8 * (x0 + dx), y0 + dy, 0, zsrc, 0);
+        else tc::tma_load_5d(dst, map, bar, 0, x0 + dx, y0 + dy, 0, zsrc);
+        return;
+    }
+    const int plane_bytes = g.box_x * g.box_y * 16;
+    for (int zz = 0; zz < g.box_z; ++zz) {
+        const int zn = z0 + zz, z = zn % g.D + dz;
+        const int zsrc = zn < g.NZ && z >= 0 && z < g.D ? zn + dz : -1;
+        for (int cg = 0; cg < NCG; ++cg) {
+            uint8_t *d = dst + cg * 2048 + zz * plane_bytes;
+            if (rows) tc::tma_load_5d(d, map, bar, 8 * (x0 + dx), y0 + dy, cg, zsrc, 0);
+            else tc::tma_load_5d(d, map, bar, 0, x0 + dx, y0 + dy, cg, zsrc);
+        }
+    }
+}
+
 template <int CIN, int COUT>
 struct ConvSmem {
     static constexpr int A_BYTES = 128 * CIN * 2;
@@ -84,18 +113,7 @@ conv3d_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __nv_bfloat16 *
             }
             uint8_t *a = smem + s * S::STAGE;
             tc::mbar_arrive_expect_tx(&full[s], S::A_BYTES + S::B_BYTES);
-            if (!multi) {
-                tc::tma_load_5d(a, &xmap, &full[s], 0, x0 + dx, y0 + dy, 0, z0 + dz);
-            } else {
-                const int plane_bytes = g.box_x * g.box_y * 16;
-                for (int zz = 0; zz < g.box_z; ++zz) {
-                    const int zn = z0 + zz, zi = zn % g.D;
-                    const int zsrc = (zn < g.NZ && zi + dz >= 0 && zi + dz < g.D) ? zn + dz : -1;
-                    for (int cg = 0; cg < CIN / 8; ++cg)
-                        tc::tma_load_5d(a + cg * 2048 + zz * plane_bytes, &xmap, &full[s], 0, x0 + dx, y0 + dy, cg,
-                                        zsrc);
-                }
-            }
+            load_tile<CIN / 8>(a, &xmap, &full[s], g, x0, y0, z0, dx, dy, dz);
             tc::bulk_load(a + S::A_BYTES, wpack + (size_t)tap * COUT * CIN, S::B_BYTES, &full[s]);
             ++it;
         }
@@ -219,8 +237,6 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant_
     const int ntiles = g.tiles_x * g.tiles_y * g.tiles_z;
     const int t_begin = blockIdx.x * tiles_per_cta;
     const int t_end = min(ntiles, t_begin + tiles_per_cta);
-    const bool multi = g.box_z > 1;
-    const int plane_bytes = g.box_x * g.box_y * 16;
 
     // rows of a partial last group read stale stage bytes: start them as zeros
     for (int q = threadIdx.x; q < S::STAGES * S::STAGE / 16; q += CONV_THREADS)
@@ -269,30 +285,9 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant_
                     const int tap = tap0 + q;
                     const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
                     uint8_t *dst = a + q * (CIN / 8) * 2048;
-                    if (!multi) {
-                        const int z = z0 % g.D;
-                        const int zsrc = (z + dz >= 0 && z + dz < g.D) ? z0 + dz : -1;
-                        tc::tma_load_5d(dst, &xmap, &full[s], 0, x0 + dx, y0 + dy, 0, zsrc);
-                    } else {
-                        for (int zz = 0; zz < g.box_z; ++zz) {
-                            const int zn = z0 + zz, zi = zn % g.D;
-                            const int zsrc = (zn < g.NZ && zi + dz >= 0 && zi + dz < g.D) ? zn + dz : -1;
-                            for (int cg = 0; cg < CIN / 8; ++cg)
-                                tc::tma_load_5d(dst + cg * 2048 + zz * plane_bytes, &xmap, &full[s], 0, x0 + dx,
-                                                y0 + dy, cg, zsrc);
-                        }
-                    }
+                    load_tile<CIN / 8>(dst, &xmap, &full[s], g, x0, y0, z0, dx, dy, dz);
                 }
-                if (!multi) {
-                    tc::tma_load_5d(b, &gmap, &full[s], 0, x0, y0, 0, z0);
-                } else {
-                    for (int zz = 0; zz < g.box_z; ++zz) {
-                        const int zn = z0 + zz;
-                        for (int cg = 0; cg < COUT / 8; ++cg)
-                            tc::tma_load_5d(b + cg * 2048 + zz * plane_bytes, &gmap, &full[s], 0, x0, y0, cg,
-                                            zn < g.NZ ? zn : -1);
-                    }
-                }
+                load_tile<COUT / 8>(b, &gmap, &full[s], g, x0, y0, z0, 0, 0, 0);
             }
         }
     } else if (threadIdx.x == 32) {
@@ -479,6 +474,12 @@ gbsw_status conv_geometry(int NZ, int D, int H, int W, ConvGeom *g)
     } else if (H % by != 0) {
         return GBSW_ERR_ARG;
     }
+    // rows of at most 32 voxels, so that a box may be rows of voxels (LOAD_ROWS)
+    if (bz == 1 && bx > 32 && H % 4 == 0) {
+        bx = 32;
+        by = 4;
+    }
+    g->load = bx > 32 ? LOAD_VOXELS : bz > 1 && (D % bz == 0 || bz % D == 0) ? LOAD_SAMPLES : LOAD_ROWS;
     g->NZ = NZ;
     g->D = D;
     g->H = H;
@@ -499,12 +500,42 @@ gbsw_status conv_tensor_map(const __nv_bfloat16 *base, const ConvGeom &g, int cg
     EncodeFn fn = encode_fn();
     if (!fn) return GBSW_ERR_CUDA;
     if (((uintptr_t)base & 15) != 0) return GBSW_ERR_ARG;
-    const cuuint64_t dims[5] = {8, (cuuint64_t)g.W, (cuuint64_t)g.H, (cuuint64_t)cg_total, (cuuint64_t)g.NZ};
-    const cuuint64_t strides[4] = {16, (cuuint64_t)g.W * 16, (cuuint64_t)g.H * g.W * 16,
-                                   (cuuint64_t)cg_total * g.H * g.W * 16};
-    // one box per tap (all channel groups), or per (plane, group) for multi-plane tiles
-    const cuuint32_t box[5] = {8, (cuuint32_t)g.box_x, (cuuint32_t)g.box_y, g.box_z > 1 ? 1u : (cuuint32_t)cg_total,
-                               1};
+    const cuuint64_t W = g.W, H = g.H, D = g.D, NZ = g.NZ, cg = cg_total;
+    const cuuint64_t row = W * 16, group = H * row, plane = cg * group;  // bytes
+    const cuuint32_t bx = g.box_x, by = g.box_y, bz = g.box_z;
+    // all channel groups at once, or (plane, group) by (plane, group)
+    const cuuint32_t bcg = bz > 1 && g.load != LOAD_SAMPLES ? 1u : (cuuint32_t)cg_total;
+    cuuint64_t dims[5], strides[4];
+    cuuint32_t box[5];
+    auto set = [&](int k, cuuint64_t dim, cuuint64_t stride, cuuint32_t b) {
+        dims[k] = dim;
+        if (k > 0) strides[k - 1] = stride;
+        box[k] = b;
+    };
+    switch (g.load) {
+    case LOAD_VOXELS:
+        set(0, 8, 0, 8);
+        set(1, W, 16, bx);
+        set(2, H, row, by);
+        set(3, cg, group, bcg);
+        set(4, NZ, plane, 1);
+        break;
+    case LOAD_ROWS:
+        set(0, 8 * W, 0, 8 * bx);
+        set(1, H, row, by);
+        set(2, cg, group, bcg);
+        set(3, NZ, plane, 1);
+        set(4, 1, NZ * plane, 1);
+        break;
+    default: {
+        const cuuint32_t planes = std::min(g.D, g.box_z);
+        set(0, 8 * W, 0, 8 * bx);
+        set(1, H, row, by);
+        set(2, D, plane, planes);
+        set(3, NZ / D, D * plane, bz / planes);
+        set(4, cg, group, bcg);
+    }
+    }
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void *)base, dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,

@@ -16,7 +16,8 @@
 //
 // Small planes (box_x * H < 128, the coarse levels of a network run on a
 // coarsened grid) make a tile of box_z consecutive planes of box_y = H rows.
-// Each (plane, channel group) is then one TMA box {8, box_x, box_y, 1, 1}
+// If box_z planes are whole samples or divide one, a tile is one box per tap
+// (LOAD_SAMPLES).  Otherwise each (plane, channel group) is one TMA box
 // placed at plane * box_x * box_y * 16 bytes inside its slab, which keeps the
 // canonical layout; a plane whose tap leaves its sample, or that lies past
 // the last plane, is loaded from z = -1 (all out of bounds: zero fill) and
@@ -45,11 +46,23 @@
 
 namespace gbsw {
 
+// How the 128 voxels x Cin channels of a (shifted) tile are fetched.  A TMA
+// box costs about a cycle per innermost row, so rows are made long: with rows
+// of one voxel's 16 bytes the loads of a 16-channel tile and tap took 256
+// cycles, more than everything else in the kernels together.
+enum ConvLoad : int {
+    LOAD_VOXELS = 0,   // rows of 8 channels; map {8, W, H, C/8, NZ}, one box per tap
+    LOAD_ROWS = 1,     // rows of box_x voxels (<= 32: a box is at most 256 elements wide); map {8W, H, C/8, NZ, 1}
+    LOAD_SAMPLES = 2   // small planes, tiles of whole samples or whole parts of one: map {8W, H, D, N, C/8},
+                       // one box per tap; planes outside a sample are zero fill
+};
+
 struct ConvGeom {
     int NZ, H, W;        // samples*D, rows, columns
     int D;               // depth of one sample
     int box_x, box_y;    // tile = box_z planes x box_y rows x box_x voxels = 128 voxels
     int box_z;           // 1 unless box_x * H < 128
+    int load;            // ConvLoad: how a tile is fetched
     int tiles_x, tiles_y, tiles_z;
     int out_cg_total, out_cg0;    // output tensor channel groups and offset
     int mask_cg_total, mask_cg0;  // mask tensor (EPI_MASK)
