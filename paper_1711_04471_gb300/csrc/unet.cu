@@ -203,13 +203,13 @@ gbsw_status get_acts(gbsw_unet *u, int N, int D, int H, int W, bool train, Acts 
 gbsw_status repack(gbsw_unet *u, cudaStream_t s)
 {
     if (!u->packs_dirty) return GBSW_OK;
-    TRY(pack_weights_padded(u->params + u->w_off[L1A], LAYERS[L1A].cin, 16, LAYERS[L1A].cout, 0, u->pack_fwd[L1A], s));
+    PackList list{};
+    list.add(u->params + u->w_off[L1A], LAYERS[L1A].cin, 16, LAYERS[L1A].cout, 0, u->pack_fwd[L1A]);
     for (int l = 1; l < NLAYERS; ++l) {
-        gbsw_status st = pack_weights(u->params + u->w_off[l], LAYERS[l].cin, LAYERS[l].cout, 0, u->pack_fwd[l], s);
-        if (st == GBSW_OK)
-            st = pack_weights(u->params + u->w_off[l], LAYERS[l].cin, LAYERS[l].cout, 1, u->pack_bwd[l], s);
-        if (st != GBSW_OK) return st;
+        list.add(u->params + u->w_off[l], LAYERS[l].cin, LAYERS[l].cin, LAYERS[l].cout, 0, u->pack_fwd[l]);
+        list.add(u->params + u->w_off[l], LAYERS[l].cin, LAYERS[l].cin, LAYERS[l].cout, 1, u->pack_bwd[l]);
     }
+    TRY(pack_weights(list, s));
     u->packs_dirty = false;
     return GBSW_OK;
 }

@@ -77,7 +77,9 @@ extern "C" gbsw_status unet_conv3d(int nsamples, int D, int H, int W, int cin, i
         CHK(to_blocked(mask, g.NZ, H, W, cout, mb, cout / 8, 0, s));
     }
     CHK(to_blocked(x, g.NZ, H, W, cin, xb, cin_k / 8, 0, s));
-    CHK(pack_weights_padded(w, cin, cin_k, cout, 0, wp, s));
+    PackList packs{};
+    packs.add(w, cin, cin_k, cout, 0, wp);
+    CHK(pack_weights(packs, s));
     ConvCall c{};
     CHK(conv_tensor_map(xb, g, cin_k / 8, &c.xmap));
     g.mask_cg_total = cout / 8;

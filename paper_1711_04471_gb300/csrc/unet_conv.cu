@@ -14,36 +14,53 @@ namespace gbsw {
 
 namespace {
 
-constexpr int CONV_STAGES = 4;
 constexpr int CONV_THREADS = 128;
 
 __device__ __forceinline__ void set_status(int *status, int code) { atomicCAS(status, DEV_OK, code); }
 
-// Thread 0: the tile at (x0, y0, z0) shifted by (dx, dy, dz), NCG channel
-// groups, into slabs of 2048 bytes at dst (128 * NCG * 16 bytes arrive on bar).
-template <int NCG>
-__device__ __forceinline__ void load_tile(uint8_t *dst, const CUtensorMap *map, uint64_t *bar, const ConvGeom &g, int x0,
-                                          int y0, int z0, int dx, int dy, int dz)
+// Where a tile lies: z0 = sample * D + z.
+struct TilePos {
+    int x0, y0, z0, sample, z;
+};
+
+__device__ __forceinline__ TilePos tile_pos(const ConvGeom &g, int t)
 {
+    TilePos p;
+    p.x0 = (t % g.tiles_x) * g.box_x;
+    t /= g.tiles_x;
+    p.y0 = (t % g.tiles_y) * g.box_y;
+    p.z0 = (t / g.tiles_y) * g.box_z;
+    p.sample = p.z0 / g.D;
+    p.z = p.z0 - p.sample * g.D;
+    return p;
+}
+
+// One thread: the tile at p shifted by (dx, dy, dz), NCG channel groups,
+// into slabs of 2048 bytes at dst (128 * NCG * 16 bytes arrive on bar).
+template <int NCG>
+__device__ __forceinline__ void load_tile(uint8_t *dst, const CUtensorMap *map, uint64_t *bar, const ConvGeom &g,
+                                          const TilePos &p, int dx, int dy, int dz)
+{
+    const int x = p.x0 + dx, y = p.y0 + dy, z = p.z + dz;
     if (g.load == LOAD_SAMPLES) {
-        tc::tma_load_5d(dst, map, bar, 8 * dx, dy, z0 % g.D + dz, z0 / g.D, 0);
+        tc::tma_load_5d(dst, map, bar, 8 * x, y, z, p.sample, 0);
         return;
     }
     const bool rows = g.load == LOAD_ROWS;
     if (g.box_z == 1) {
-        const int z = z0 % g.D + dz, zsrc = z >= 0 && z < g.D ? z0 + dz : -1;
-        if (rows) tc::tma_load_5d(dst, map, bar, 8 * (x0 + dx), y0 + dy, 0, zsrc, 0);
-        else tc::tma_load_5d(dst, map, bar, 0, x0 + dx, y0 + dy, 0, zsrc);
+        const int zsrc = z >= 0 && z < g.D ? p.z0 + dz : -1;
+        if (rows) tc::tma_load_5d(dst, map, bar, 8 * x, y, 0, zsrc, 0);
+        else tc::tma_load_5d(dst, map, bar, 0, x, y, 0, zsrc);
         return;
     }
     const int plane_bytes = g.box_x * g.box_y * 16;
     for (int zz = 0; zz < g.box_z; ++zz) {
-        const int zn = z0 + zz, z = zn % g.D + dz;
-        const int zsrc = zn < g.NZ && z >= 0 && z < g.D ? zn + dz : -1;
+        const int zn = p.z0 + zz, zi = zn % g.D + dz;
+        const int zsrc = zn < g.NZ && zi >= 0 && zi < g.D ? zn + dz : -1;
         for (int cg = 0; cg < NCG; ++cg) {
             uint8_t *d = dst + cg * 2048 + zz * plane_bytes;
-            if (rows) tc::tma_load_5d(d, map, bar, 8 * (x0 + dx), y0 + dy, cg, zsrc, 0);
-            else tc::tma_load_5d(d, map, bar, 0, x0 + dx, y0 + dy, cg, zsrc);
+            if (rows) tc::tma_load_5d(d, map, bar, 8 * x, y, cg, zsrc, 0);
+            else tc::tma_load_5d(d, map, bar, 0, x, y, cg, zsrc);
         }
     }
 }
@@ -53,8 +70,13 @@ struct ConvSmem {
     static constexpr int A_BYTES = 128 * CIN * 2;
     static constexpr int B_BYTES = COUT * CIN * 2;
     static constexpr int STAGE = ((A_BYTES + B_BYTES + 1023) / 1024) * 1024;
-    static constexpr int BAR_OFF = CONV_STAGES * STAGE;
-    static constexpr int BYTES = BAR_OFF + 128 + 1024;  // barriers + TMEM slot, plus alignment slack
+    // Taps in flight.  Four leave room for more tiles per SM, whose epilogues
+    // overlap; with few tiles only the ring hides the loads' latency
+    // (16 -> 16 channels: 8192 tiles 75 us with 4, 111 with 9; 64 -> 32, 8 tiles
+    // 13.9 with 4, 12.7 with 9).
+    static constexpr int STAGES = 4;
+    static constexpr int DEEP = 9 * STAGE <= 200 * 1024 ? 9 : 200 * 1024 / STAGE;
+    static constexpr int bytes(int stages) { return stages * STAGE + 256 + 1024; }  // barriers + TMEM slot, alignment slack
     static constexpr int TMEM_COLS = COUT < 32 ? 32 : COUT;
 };
 
@@ -62,33 +84,29 @@ template <int CIN, int COUT>
 __global__ void __launch_bounds__(CONV_THREADS)
 conv3d_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __nv_bfloat16 *__restrict__ wpack,
                  const float *__restrict__ bias, __nv_bfloat16 *__restrict__ y, float *__restrict__ y_f32,
-                 const __nv_bfloat16 *__restrict__ mask, ConvGeom g, int epi, int *status)
+                 const __nv_bfloat16 *__restrict__ mask, ConvGeom g, int epi, int stages, int *status)
 {
     using S = ConvSmem<CIN, COUT>;
     static_assert(CIN % 16 == 0 && COUT % 16 == 0 && COUT <= 256, "UMMA shape");
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint64_t *full = (uint64_t *)(smem + S::BAR_OFF);
-    uint64_t *empty = full + CONV_STAGES;
-    uint64_t *done = empty + CONV_STAGES;
+    uint64_t *full = (uint64_t *)(smem + stages * S::STAGE);
+    uint64_t *empty = full + stages;
+    uint64_t *done = empty + stages;
     uint32_t *tmem_slot = (uint32_t *)(done + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int t = blockIdx.x;
-    const int tx = t % g.tiles_x;
-    t /= g.tiles_x;
-    const int ty = t % g.tiles_y;
-    const int tz = t / g.tiles_y;
-    const int x0 = tx * g.box_x, y0 = ty * g.box_y, z0 = tz * g.box_z;
+    const TilePos pos = tile_pos(g, blockIdx.x);
+    // the taps of a single-plane tile that stay in the sample: a range
     const bool multi = g.box_z > 1;  // tile of several planes (small planes)
-    const int z = z0 % g.D;          // the plane of a single-plane tile
+    const int tap_begin = !multi && pos.z == 0 ? 9 : 0, tap_end = !multi && pos.z == g.D - 1 ? 18 : 27;
 
     if (warp == 0) {
         tc::tmem_alloc(tmem_slot, S::TMEM_COLS);
         tc::tmem_relinquish();
     }
     if (threadIdx.x == 32) {
-        for (int s = 0; s < CONV_STAGES; ++s) {
+        for (int s = 0; s < stages; ++s) {
             tc::mbar_init(&full[s], 1);
             tc::mbar_init(&empty[s], 1);
         }
@@ -101,34 +119,36 @@ conv3d_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __nv_bfloat16 *
     const uint32_t tmem = *tmem_slot;
 
     if (threadIdx.x == 0) {
-        // producer: one stage per valid tap
-        int it = 0;
-        for (int tap = 0; tap < 27; ++tap) {
-            const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-            if (!multi && (z + dz < 0 || z + dz >= g.D)) continue;
-            const int s = it % CONV_STAGES;
-            if (it >= CONV_STAGES && !tc::mbar_wait(&empty[s], ((it / CONV_STAGES) - 1) & 1)) {
+        // producer: one stage per tap
+        int dx = -1, dy = -1, dz = tap_begin / 9 - 1, s = 0, parity = 1;
+        for (int tap = tap_begin; tap < tap_end; ++tap) {
+            // the first round passes: an empty stage's preceding phase is complete
+            if (!tc::mbar_wait(&empty[s], parity)) {
                 set_status(status, DEV_TIMEOUT);
                 break;
             }
             uint8_t *a = smem + s * S::STAGE;
             tc::mbar_arrive_expect_tx(&full[s], S::A_BYTES + S::B_BYTES);
-            load_tile<CIN / 8>(a, &xmap, &full[s], g, x0, y0, z0, dx, dy, dz);
+            load_tile<CIN / 8>(a, &xmap, &full[s], g, pos, dx, dy, dz);
             tc::bulk_load(a + S::A_BYTES, wpack + (size_t)tap * COUT * CIN, S::B_BYTES, &full[s]);
-            ++it;
+            if (++s == stages) {
+                s = 0;
+                parity ^= 1;
+            }
+            if (++dx == 2) {
+                dx = -1;
+                if (++dy == 2) {
+                    dy = -1;
+                    ++dz;
+                }
+            }
         }
     } else if (threadIdx.x == 32) {
         // MMA issuer
         constexpr uint32_t idesc = tc::idesc_bf16_f32(128, COUT);
-        int it = 0;
-        bool ok = true;
-        for (int tap = 0; tap < 27 && ok; ++tap) {
-            const int dz = tap / 9 - 1;
-            if (!multi && (z + dz < 0 || z + dz >= g.D)) continue;
-            const int s = it % CONV_STAGES;
-            if (!tc::mbar_wait(&full[s], (it / CONV_STAGES) & 1)) {
+        for (int it = 0, s = 0, parity = 0; it < tap_end - tap_begin; ++it) {
+            if (!tc::mbar_wait(&full[s], parity)) {
                 set_status(status, DEV_TIMEOUT);
-                ok = false;
                 break;
             }
             tc::fence_after_sync();
@@ -141,7 +161,10 @@ conv3d_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __nv_bfloat16 *
                 tc::umma_bf16(tmem, ad, bd, idesc, (it > 0 || kc > 0) ? 1u : 0u);
             }
             tc::umma_commit(&empty[s]);
-            ++it;
+            if (++s == stages) {
+                s = 0;
+                parity ^= 1;
+            }
         }
         tc::umma_commit(done);
     }
@@ -153,8 +176,8 @@ conv3d_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __nv_bfloat16 *
     tc::fence_after_sync();
     const int m = warp * 32 + lane;
     const int plane = g.box_x * g.box_y;
-    const int zn = z0 + m / plane, r = m % plane;
-    const int yy = y0 + r / g.box_x, xx = x0 + r % g.box_x;
+    const int zn = pos.z0 + m / plane, r = m % plane;
+    const int yy = pos.y0 + r / g.box_x, xx = pos.x0 + r % g.box_x;
     const bool stored = zn < g.NZ;  // false only past the last plane of a multi-plane tile
 #pragma unroll
     for (int cb = 0; cb < COUT / 8; ++cb) {
@@ -212,7 +235,7 @@ struct WgradSmem {
 
 // dW[tap][co][ci] += sum over the voxels of tiles [t_begin, t_end) of
 // gz[v][co] x[v + off(tap)][ci] (zero outside the sample), one CTA per
-// chunk of tiles.  Per tile and tap group: thread 0 loads the group's
+// chunk of tiles.  Per tile and tap group: warp 0 loads the group's
 // shifted x tiles (the forward conv's TMA boxes; a plane whose tap leaves
 // its sample, or past the last plane, is loaded from z = -1, all zero
 // fill) and the gz tile into a stage; thread 32 issues 8 MMAs (M = 128
@@ -259,35 +282,29 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant_
     tc::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
 
-    if (threadIdx.x == 0) {
-        // producer
+    if (warp == 0) {
+        // producers: a lane per tap of the group, and one for the gz tile
         int it = 0;
         bool ok = true;
         for (int t = t_begin; t < t_end && ok; ++t) {
-            int tt = t;
-            const int x0 = (tt % g.tiles_x) * g.box_x;
-            tt /= g.tiles_x;
-            const int y0 = (tt % g.tiles_y) * g.box_y;
-            const int z0 = (tt / g.tiles_y) * g.box_z;
+            const TilePos pos = tile_pos(g, t);
             for (int gi = 0; gi < S::NGROUPS; ++gi, ++it) {
                 const int s = it % S::STAGES;
-                if (it >= S::STAGES && !tc::mbar_wait(&empty[s], ((it / S::STAGES) - 1) & 1)) {
-                    set_status(status, DEV_TIMEOUT);
-                    ok = false;
-                    break;
+                const int tap = gi * S::TPG + lane, ntap = min(S::TPG, 27 - gi * S::TPG);
+                if (lane == 0) {
+                    ok = it < S::STAGES || tc::mbar_wait(&empty[s], ((it / S::STAGES) - 1) & 1);
+                    if (ok) tc::mbar_arrive_expect_tx(&full[s], ntap * CIN * 256 + COUT * 256);
+                    else set_status(status, DEV_TIMEOUT);
                 }
-                const int tap0 = gi * S::TPG;
-                const int ntap = min(S::TPG, 27 - tap0);
+                ok = __shfl_sync(0xffffffffu, ok, 0);
+                if (!ok) break;
                 uint8_t *a = smem + s * S::STAGE;
-                uint8_t *b = a + S::A_BYTES;
-                tc::mbar_arrive_expect_tx(&full[s], ntap * CIN * 256 + COUT * 256);
-                for (int q = 0; q < ntap; ++q) {
-                    const int tap = tap0 + q;
-                    const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-                    uint8_t *dst = a + q * (CIN / 8) * 2048;
-                    load_tile<CIN / 8>(dst, &xmap, &full[s], g, x0, y0, z0, dx, dy, dz);
-                }
-                load_tile<COUT / 8>(b, &gmap, &full[s], g, x0, y0, z0, 0, 0, 0);
+                if (lane < ntap)
+                    load_tile<CIN / 8>(a + lane * (CIN / 8) * 2048, &xmap, &full[s], g, pos, tap % 3 - 1,
+                                       (tap / 3) % 3 - 1, tap / 9 - 1);
+                else if (lane == 31)
+                    load_tile<COUT / 8>(a + S::A_BYTES, &gmap, &full[s], g, pos, 0, 0, 0);
+                __syncwarp();
             }
         }
     } else if (threadIdx.x == 32) {
@@ -348,25 +365,30 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant_
 // flip = 1 the weights of the backward-data convolution:
 // pack[tap][co/8][ci][co%8] = w[26 - tap][co][ci].  The source holds
 // cin_src <= cin input channels per (tap, co); the forward pack's channels
-// ci >= cin_src are zero (a zero-padded input).
-__global__ void conv_pack_kernel(const float *__restrict__ w, int cin_src, int cin, int cout, int flip,
-                                 __nv_bfloat16 *__restrict__ pack)
+// ci >= cin_src are zero (a zero-padded input).  One launch makes all packs
+// of the list (a network's 15 launches of 3 us were 5 % of a small training
+// step); block b belongs to the job with first_block <= b.
+__global__ void conv_pack_kernel(const __grid_constant__ PackList list)
 {
+    int j = 0;
+    while (j + 1 < list.n && (int)blockIdx.x >= list.job[j + 1].first_block) ++j;
+    const PackJob &job = list.job[j];
+    const int cin = job.cin, cout = job.cout;
     const int n = 27 * cin * cout;
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    const int q = (blockIdx.x - job.first_block) * blockDim.x + threadIdx.x;
     if (q >= n) return;
     const int tap = q / (cin * cout);
     const int r = q % (cin * cout);
     const int co = r / cin, ci = r % cin;
-    const float v = ci < cin_src ? w[((size_t)tap * cout + co) * cin_src + ci] : 0.0f;
+    const float v = ci < job.cin_src ? job.w[((size_t)tap * cout + co) * job.cin_src + ci] : 0.0f;
     size_t dst;
-    if (!flip) {
+    if (!job.flip) {
         dst = (((size_t)tap * (cin / 8) + ci / 8) * cout + co) * 8 + ci % 8;
     } else {
         const int tp = 26 - tap;  // the packed conv has Cin' = cout, Cout' = cin
         dst = (((size_t)tp * (cout / 8) + co / 8) * cin + ci) * 8 + co % 8;
     }
-    pack[dst] = __float2bfloat16_rn(v);
+    job.pack[dst] = __float2bfloat16_rn(v);
 }
 
 // dense FP32 (zn, y, x, C) <-> C8-blocked BF16
@@ -426,12 +448,13 @@ gbsw_status launch_conv_t(const ConvCall &c, cudaStream_t s)
     static bool configured = false;
     if (!configured) {
         GBSW_CUDA_TRY(cudaFuncSetAttribute(conv3d_tc_kernel<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           S::BYTES));
+                                           S::bytes(S::DEEP)));
         configured = true;
     }
     const int ntiles = c.geom.tiles_z * c.geom.tiles_y * c.geom.tiles_x;
-    conv3d_tc_kernel<CIN, COUT><<<ntiles, CONV_THREADS, S::BYTES, s>>>(c.xmap, c.wpack, c.bias, c.y, c.y_f32, c.mask,
-                                                                       c.geom, c.epi, c.status);
+    const int stages = ntiles <= sm_count() ? S::DEEP : S::STAGES;
+    conv3d_tc_kernel<CIN, COUT><<<ntiles, CONV_THREADS, S::bytes(stages), s>>>(
+        c.xmap, c.wpack, c.bias, c.y, c.y_f32, c.mask, c.geom, c.epi, stages, c.status);
     GBSW_LAUNCH_CHECK();
     return GBSW_OK;
 }
@@ -574,19 +597,26 @@ gbsw_status launch_wgrad_tc(int cin, int cout, const WgradCall &c, cudaStream_t 
     return GBSW_ERR_ARG;
 }
 
-gbsw_status pack_weights(const float *w, int cin, int cout, int flip, __nv_bfloat16 *pack, cudaStream_t s)
+gbsw_status pack_weights(PackList list, cudaStream_t s)
 {
-    return pack_weights_padded(w, cin, cin, cout, flip, pack, s);
-}
-
-gbsw_status pack_weights_padded(const float *w, int cin_src, int cin, int cout, int flip, __nv_bfloat16 *pack,
-                                cudaStream_t s)
-{
-    if (cin_src < 1 || cin_src > cin || (flip && cin_src != cin)) return GBSW_ERR_ARG;
-    const int n = 27 * cin * cout;
-    conv_pack_kernel<<<ceil_div(n, 256), 256, 0, s>>>(w, cin_src, cin, cout, flip, pack);
+    if (list.n < 1 || list.n > PackList::MAX) return GBSW_ERR_ARG;
+    int blocks = 0;
+    for (int j = 0; j < list.n; ++j) {
+        PackJob &job = list.job[j];
+        if (job.cin_src < 1 || job.cin_src > job.cin || (job.flip && job.cin_src != job.cin)) return GBSW_ERR_ARG;
+        job.first_block = blocks;
+        blocks += ceil_div(27 * job.cin * job.cout, 256);
+    }
+    conv_pack_kernel<<<blocks, 256, 0, s>>>(list);
     GBSW_LAUNCH_CHECK();
     return GBSW_OK;
+}
+
+gbsw_status pack_weights(const float *w, int cin, int cout, int flip, __nv_bfloat16 *pack, cudaStream_t s)
+{
+    PackList list{};
+    list.add(w, cin, cin, cout, flip, pack);
+    return pack_weights(list, s);
 }
 
 gbsw_status to_blocked(const float *src, int NZ, int H, int W, int C, __nv_bfloat16 *dst, int cg_total, int cg0,

@@ -25,10 +25,10 @@
 //
 // One CTA computes one tile of 128 voxels (box_z x box_y x box_x) and
 // all Cout channels: thread 0 of warp 0 issues the loads of tap t into a
-// 4-stage ring, thread 0 of warp 1 issues Cin/16 MMAs (M=128, N=Cout, K=16)
-// per tap and commits each stage back to the producer, and all four warps
-// read the accumulator (warp w owns TMEM lanes 32w..32w+31 = voxels) for
-// the epilogue.
+// ring of stages, thread 0 of warp 1 issues Cin/16 MMAs (M=128, N=Cout,
+// K=16) per tap and commits each stage back to the producer, and all four
+// warps read the accumulator (warp w owns TMEM lanes 32w..32w+31 = voxels)
+// for the epilogue.
 //
 // Weight gradients (wgrad_tc_kernel) contract over voxels instead:
 // dW[tap][co][ci] = sum_v gz[v][co] x[v + off(tap)][ci].  The same
