@@ -75,7 +75,8 @@ struct ConvSmem {
     // (16 -> 16 channels: 8192 tiles 75 us with 4, 111 with 9; 64 -> 32, 8 tiles
     // 13.9 with 4, 12.7 with 9).
     static constexpr int STAGES = 4;
-    static constexpr int DEEP = 9 * STAGE <= 200 * 1024 ? 9 : 200 * 1024 / STAGE;
+    static constexpr int FIT = 72 * 1024 / STAGE;  // what leaves room for a weight-gradient CTA on the SM
+    static constexpr int DEEP = FIT > 9 ? 9 : FIT < STAGES ? STAGES : FIT;
     static constexpr int bytes(int stages) { return stages * STAGE + 256 + 1024; }  // barriers + TMEM slot, alignment slack
     static constexpr int TMEM_COLS = COUT < 32 ? 32 : COUT;
 };
