@@ -1015,10 +1015,14 @@ __device__ __noinline__ void sort_test(const SorTileRun &run, bool counting, int
         c.status = DEV_OK;
         c.bb = bb;
     }
+    const double rr_prev = c.rr;  // of the check before, `ran` iterations ago
     c.rr = rr;
-    // far from the tolerance, and no prediction that needs the norm: no root, no division (a few us in FP64)
+    // Far from the tolerance: no root, no logarithm, no division (a few us in
+    // FP64).  A prediction then has no say if the tolerance is more than m
+    // iterations away: tol / rho < rho / rho_prev over at least m iterations.
     if (counting && !run.fixed && (run.chunk == 0 || run.chunk >= run.m) && isfinite(rr) && c.bb >= 1e-60 &&
-        rr > c.bb * run.tol2_above && c.iters < run.max_iter) {
+        rr > c.bb * run.tol2_above && c.iters < run.max_iter &&
+        (run.chunk == 0 || rr * rr > run.tol2_above * rr_prev * c.bb * (1.0 + 1e-9))) {
         c.next = run.chunk > 0 ? run.chunk : run.m;
         return;
     }
@@ -1030,8 +1034,9 @@ __device__ __noinline__ void sort_test(const SorTileRun &run, bool counting, int
     const bool done = bad || c.bb < 1e-60 || rho <= run.tol || c.iters >= most;
     c.done = done ? 1 : 0;
     int next = run.m;
-    if (run.chunk > 0 && counting && !done && rho > 0.0 && rho < c.rho_prev && c.iters > c.iters_prev) {
-        const double lg = log(rho / c.rho_prev) / (double)(c.iters - c.iters_prev);
+    const double rho_prev = c.bb > 0.0 ? sqrt(rr_prev / c.bb) : 0.0;
+    if (run.chunk > 0 && counting && !done && rho > 0.0 && rho < rho_prev && ran > 0) {
+        const double lg = log(rho / rho_prev) / (double)ran;
         const double n = log(run.tol / rho) / lg;
         if (n < (double)run.m) next = max(1, (int)ceil(1.03 * n) + 1);
     }
@@ -1039,8 +1044,6 @@ __device__ __noinline__ void sort_test(const SorTileRun &run, bool counting, int
     if (run.fixed) c.next = counting ? 0 : run.n;
     else if (done) c.next = 0;
     else c.next = run.chunk > 0 ? run.chunk * ((next + run.chunk - 1) / run.chunk) : run.m;
-    c.rho_prev = rho;
-    c.iters_prev = c.iters;
 }
 
 // Cooperative launch: grid py * pz, block plan.threads.  I = 0: a tile of
