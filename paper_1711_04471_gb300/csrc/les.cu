@@ -68,7 +68,10 @@ __device__ __forceinline__ long long L(const PDims &d, int i, int j, int k)
 // ((nz+2) planes); always true in the product build.
 #define LES_OK(d, c) GBSW_INBOUNDS((c), (long long)(d).plane * ((d).nz + 2), &g_les_bounds)
 
-// velnw: projection with the previous pressure, interior faces only.
+// velnw: projection with the previous pressure, interior faces only.  Bound
+// by the FP64 pipe: three differences per cell; their conversions to FP32 are
+// integer operations (with them on the FP64 pipe too a launch at 300x300x90
+// took 113 us).
 __global__ void les_velnw_kernel(LDev q, const double *__restrict__ p, float *__restrict__ u, float *__restrict__ v,
                                  float *__restrict__ w)
 {
@@ -81,9 +84,9 @@ __global__ void les_velnw_kernel(LDev q, const double *__restrict__ p, float *__
     const double pc = p[c];
     const double pe = (i < d.nx) ? p[c + 1] : -pc;
     const double pn = p[cn];
-    u[c] -= q.c_grad * (float)(pe - pc);
-    v[c] -= q.c_grad * (float)(pn - pc);
-    if (k < d.nz) w[c] -= q.c_grad * (float)(p[c + d.plane] - pc);
+    u[c] -= q.c_grad * f32_from_f64(pe - pc);
+    v[c] -= q.c_grad * f32_from_f64(pn - pc);
+    if (k < d.nz) w[c] -= q.c_grad * f32_from_f64(p[c + d.plane] - pc);
 }
 
 // ---------------------------------------------------------------- fused predictor
