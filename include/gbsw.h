@@ -147,7 +147,11 @@ gbsw_status sw_create(const gbsw_sw_params *params, const double *H, const doubl
                       void *stream, gbsw_sw **out);
 
 /* Advance the state by nsteps >= 0 time steps.  Asynchronous on the
- * context stream; several steps are fused per kernel launch. */
+ * context stream; several steps are fused per kernel launch.  With the
+ * automatic tiling a grid that fits in the SMs' registers and shared memory
+ * takes all steps of the call in one cooperative launch (not while the
+ * stream is being captured); its bounded waits between SMs report
+ * GBSW_ERR_TIMEOUT at the next sw_volume or sw_get_state. */
 gbsw_status sw_step(gbsw_sw *sw, int nsteps);
 
 /*
@@ -172,11 +176,12 @@ gbsw_status sw_get_state(gbsw_sw *sw, float *eta, float *u, float *v, uint8_t *w
 gbsw_status sw_set_state(gbsw_sw *sw, const float *eta, const float *u, const float *v);
 
 /* Number of time steps fused per kernel launch (temporal blocking depth):
- * 0 = automatic, else 1..6 (the row-segment height returns to automatic). */
+ * 0 = automatic (2 below 1.4 million cells, else 3), else 1..6 (the row-segment height returns to automatic). */
 gbsw_status sw_set_blocking(gbsw_sw *sw, int steps_per_launch);
 
-/* Tiling of the fused kernel: steps per launch (0 = automatic, else 1..6)
- * and the row-segment height of a thread block of the streaming kernel (0 =
+/* Tiling of the fused kernel: steps per launch (0 = automatic, else 1..6; 0
+ * with rows = 0, the initial setting, also admits the one-launch path of
+ * sw_step) and the row-segment height of a thread block of the streaming kernel (0 =
  * automatic: one wave of resident blocks, segments of at least 8T rows),
  * or rows < 0 for the tile kernel, made for grids that fit in L2: a block
  * holds 32 columns x h rows and a 2T-cell halo in shared memory, with
@@ -192,7 +197,9 @@ gbsw_status sw_set_tiling(gbsw_sw *sw, int steps_per_launch, int rows);
  * resident blocks, and the tile kernel for T = 1..3 with 32-row tiles and
  * with the tile height that spreads its blocks most evenly over the SMs,
  * keeps the fastest (written to *T_out, *rows_out in the encoding of
- * sw_set_tiling, if non-NULL) and restores the state exactly.  Allocates a copy of the state;
+ * sw_set_tiling, if non-NULL) and restores the state exactly.  The automatic
+ * setting's one-launch path is timed too and kept if it is faster than all
+ * of these; *T_out, *rows_out are then the fastest of the others.  Allocates a copy of the state;
  * synchronous.  The paper's grids (Sec. 6.2: 500^2 to 2000^2) are small
  * enough to stay in L2, where the best tiling differs from the 4096^2
  * default. */
@@ -205,7 +212,7 @@ void sw_destroy(gbsw_sw *sw);
  * 2DSW in FP64 end to end (Sec. 6.2: the time loop of "dyn" and "shapiro",
  * which the paper's compiler turns into three map kernels; the paper does
  * not state the precision).  The same method, parameters and conventions
- * as sw_* above, run as three kernels per step (momentum on the faces,
+ * as sw_* above, run as kernels per step (momentum and fluxes on the faces,
  * continuity on the cells, masked Shapiro filter) with every FP64
  * operation in the order written in the formulas above and rounded as
  * written (no multiply-add contraction), so the state is a deterministic
@@ -268,12 +275,15 @@ gbsw_status sw_batch_volumes(gbsw_sw_batch *b, double *volumes, double *wet_volu
 /* Copy instance m's state to host buffers in the layout of sw_get_state. */
 gbsw_status sw_batch_get_state(gbsw_sw_batch *b, int m, float *eta, float *u, float *v);
 
-/* Tiling: fused steps per level (1..4) and rows per work item (8..65536). */
+/* Tiling: fused steps per level (1..4) and rows per work item (8..65536).
+ * Until one is set or tuned, sw_batch_step picks the rows from the instances'
+ * sizes; get_tiling then reports 3, 128. */
 gbsw_status sw_batch_set_tiling(gbsw_sw_batch *b, int steps_per_level, int rows_per_item);
 gbsw_status sw_batch_get_tiling(gbsw_sw_batch *b, int *steps_per_level, int *rows_per_item);
 
 /* Time every (steps_per_level, rows_per_item) candidate on this batch
- * (state saved and restored), keep the fastest and return it.  If
+ * (state saved and restored), keep the fastest and return it; the rows
+ * picked from the sizes are timed too and kept if they are faster still.  If
  * cache_path is not NULL the choice is looked up in / appended to that
  * text file, keyed by device name and instance sizes. */
 gbsw_status sw_batch_autotune(gbsw_sw_batch *b, int trial_steps, const char *cache_path, int *steps_per_level,

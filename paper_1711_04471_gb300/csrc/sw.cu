@@ -281,7 +281,9 @@ size_t chip_smem(int per) { return ((size_t)SWC_ARRAYS * per * SWC_THREADS + 2 *
 // The cut of the grid for sw_chip_kernel: of all tiles and depths T that fit
 // the one with the least estimated cycles per step: 2000 for an exchange (none
 // with one tile), and per step 300 of latency and 650 for each cell of a
-// thread (measured: 500x500 4200 cycles, 700x700 7400).
+// thread (measured: 500x500 4200 cycles, 700x700 7400).  Several tiles exchange
+// after two steps at the earliest: with an exchange in every step the launches
+// are faster (us per step, chip and launches: 900x900 7.1, 6.4; 1100x1020 11.8, 7.6).
 SWChipPlan chip_plan(int nx, int ny)
 {
     SWChipPlan best{};
@@ -299,7 +301,7 @@ SWChipPlan chip_plan(int nx, int ny)
             if (ceil_div(nx, tw) != cx) continue;  // the same tiles as with fewer columns
             for (int cy = 1; cy <= std::min(sms / cx, ny); ++cy) {
                 const int th = ceil_div(ny, cy);
-                if (ceil_div(ny, th) != cy) continue;
+                if (ceil_div(ny, th) != cy || (T == 1 && cx * cy > 1)) continue;
                 const long long cells = (long long)(tw + 4 * T) * (th + 4 * T);
                 const int per = ceil_div(cells, SWC_THREADS);
                 if (per > SWC_MAX_PER || tw + 4 * T >= SWC_GUARD) continue;
@@ -375,7 +377,10 @@ bool capturing(const gbsw_sw *s)
     return st != cudaStreamCaptureStatusNone;
 }
 
-int auto_blocking(const gbsw_sw *) { return 3; }
+// Default depth of the launches: with few rows per segment the shorter
+// pipeline of T = 2 is better (us per step, T = 2 and 3: 500x500 4.8, 5.7;
+// 1000x1000 7.6, 7.9; 1300x1000 8.7, 8.9; 1237x1501 10.4, 9.6).
+int auto_blocking(const gbsw_sw *s) { return (long long)s->d.nx * s->d.ny < 1400000 ? 2 : 3; }
 
 int tiling_T(const gbsw_sw *s) { return s->blocking > 0 ? s->blocking : auto_blocking(s); }
 

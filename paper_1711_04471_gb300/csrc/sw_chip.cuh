@@ -24,8 +24,9 @@
 // What bounds it: the way of a word from SM to SM (about 1 us per exchange)
 // on small grids, the issue slots and shared-memory wavefronts of the phases
 // on large ones.  us per step, the kernel that the autotuner chose before,
-// this one: 100x100 1.19, 0.65; 500x500 2.55, 2.05; 700x700 5.0, 3.6;
-// 1000x1000 8.9, 7.2 (untuned, the launches took 10 us and more).
+// this one: 100x100 1.19, 0.65; 500x500 2.55, 2.05; 700x700 5.0, 3.6
+// (untuned, the launches took 10 us and more); today's launches, this one:
+// 800x800 5.9, 4.0; 900x900 6.4, 5.7.
 #pragma once
 
 #include "sw_kernels.cuh"
@@ -36,7 +37,7 @@ constexpr int SWC_THREADS = 512;
 constexpr int SWC_MAX_T = 4;
 constexpr int SWC_GUARD = 2048;        // most columns of a region
 constexpr int SWC_ARRAYS = 6;          // shared FP32 arrays of a region
-constexpr int SWC_MAX_PER = 16;        // cells per thread at most
+constexpr int SWC_MAX_PER = 14;      // cells of a thread: with 15 and 16 the registers spill and the launches are faster
 constexpr long long SWC_WAIT_CYCLES = 4000000000LL;
 
 // How a grid is cut: cx x cy tiles of tw x th cells (the last ones smaller),
