@@ -18,9 +18,9 @@ constexpr int CONV_THREADS = 128;
 
 __device__ __forceinline__ void set_status(int *status, int code) { atomicCAS(status, DEV_OK, code); }
 
-// Where a tile lies: z0 = sample * D + z.
+// Where a tile lies: z0 = sample * D + z; planes: how many of its box_z planes exist.
 struct TilePos {
-    int x0, y0, z0, sample, z;
+    int x0, y0, z0, sample, z, planes;
 };
 
 __device__ __forceinline__ TilePos tile_pos(const ConvGeom &g, int t)
@@ -29,15 +29,24 @@ __device__ __forceinline__ TilePos tile_pos(const ConvGeom &g, int t)
     p.x0 = (t % g.tiles_x) * g.box_x;
     t /= g.tiles_x;
     p.y0 = (t % g.tiles_y) * g.box_y;
-    p.z0 = (t / g.tiles_y) * g.box_z;
-    p.sample = p.z0 / g.D;
-    p.z = p.z0 - p.sample * g.D;
+    t /= g.tiles_y;
+    if (g.sample_tiles == 0) {  // whole samples: the last tile may hold fewer
+        p.z0 = t * g.box_z;
+        p.sample = p.z0 / g.D;
+        p.z = 0;
+        p.planes = g.NZ - p.z0;
+    } else {
+        p.sample = t / g.sample_tiles;
+        p.z = (t - p.sample * g.sample_tiles) * g.box_z;
+        p.z0 = p.sample * g.D + p.z;
+        p.planes = g.D - p.z;
+    }
     return p;
 }
 
-// One thread: the tile at p shifted by (dx, dy, dz), NCG channel groups,
-// into slabs of 2048 bytes at dst (128 * NCG * 16 bytes arrive on bar).
-template <int NCG>
+// One thread: the tile at p shifted by (dx, dy, dz), one box with all channel
+// groups into slabs of 2048 bytes at dst; the whole box arrives on bar, zeros
+// where it lies outside the sample.
 __device__ __forceinline__ void load_tile(uint8_t *dst, const CUtensorMap *map, uint64_t *bar, const ConvGeom &g,
                                           const TilePos &p, int dx, int dy, int dz)
 {
@@ -46,23 +55,9 @@ __device__ __forceinline__ void load_tile(uint8_t *dst, const CUtensorMap *map, 
         tc::tma_load_5d(dst, map, bar, 8 * x, y, z, p.sample, 0);
         return;
     }
-    const bool rows = g.load == LOAD_ROWS;
-    if (g.box_z == 1) {
-        const int zsrc = z >= 0 && z < g.D ? p.z0 + dz : -1;
-        if (rows) tc::tma_load_5d(dst, map, bar, 8 * x, y, 0, zsrc, 0);
-        else tc::tma_load_5d(dst, map, bar, 0, x, y, 0, zsrc);
-        return;
-    }
-    const int plane_bytes = g.box_x * g.box_y * 16;
-    for (int zz = 0; zz < g.box_z; ++zz) {
-        const int zn = p.z0 + zz, zi = zn % g.D + dz;
-        const int zsrc = zn < g.NZ && zi >= 0 && zi < g.D ? zn + dz : -1;
-        for (int cg = 0; cg < NCG; ++cg) {
-            uint8_t *d = dst + cg * 2048 + zz * plane_bytes;
-            if (rows) tc::tma_load_5d(d, map, bar, 8 * x, y, cg, zsrc, 0);
-            else tc::tma_load_5d(d, map, bar, 0, x, y, cg, zsrc);
-        }
-    }
+    const int zsrc = z >= 0 && z < g.D ? p.z0 + dz : -1;
+    if (g.load == LOAD_ROWS) tc::tma_load_5d(dst, map, bar, 8 * x, y, 0, zsrc, 0);
+    else tc::tma_load_5d(dst, map, bar, 0, x, y, 0, zsrc);
 }
 
 template <int CIN, int COUT>
@@ -130,7 +125,7 @@ conv3d_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __nv_bfloat16 *
             }
             uint8_t *a = smem + s * S::STAGE;
             tc::mbar_arrive_expect_tx(&full[s], S::A_BYTES + S::B_BYTES);
-            load_tile<CIN / 8>(a, &xmap, &full[s], g, pos, dx, dy, dz);
+            load_tile(a, &xmap, &full[s], g, pos, dx, dy, dz);
             tc::bulk_load(a + S::A_BYTES, wpack + (size_t)tap * COUT * CIN, S::B_BYTES, &full[s]);
             if (++s == stages) {
                 s = 0;
@@ -177,9 +172,9 @@ conv3d_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __nv_bfloat16 *
     tc::fence_after_sync();
     const int m = warp * 32 + lane;
     const int plane = g.box_x * g.box_y;
-    const int zn = pos.z0 + m / plane, r = m % plane;
+    const int zz = m / plane, zn = pos.z0 + zz, r = m % plane;
     const int yy = pos.y0 + r / g.box_x, xx = pos.x0 + r % g.box_x;
-    const bool stored = zn < g.NZ;  // false only past the last plane of a multi-plane tile
+    const bool stored = zz < pos.planes;  // false only past the last plane of a multi-plane tile
 #pragma unroll
     for (int cb = 0; cb < COUT / 8; ++cb) {
         float v[8];
@@ -237,9 +232,8 @@ struct WgradSmem {
 // dW[tap][co][ci] += sum over the voxels of tiles [t_begin, t_end) of
 // gz[v][co] x[v + off(tap)][ci] (zero outside the sample), one CTA per
 // chunk of tiles.  Per tile and tap group: warp 0 loads the group's
-// shifted x tiles (the forward conv's TMA boxes; a plane whose tap leaves
-// its sample, or past the last plane, is loaded from z = -1, all zero
-// fill) and the gz tile into a stage; thread 32 issues 8 MMAs (M = 128
+// shifted x tiles (the forward conv's TMA boxes; a plane outside its sample
+// is zero fill) and the gz tile into a stage; thread 32 issues 8 MMAs (M = 128
 // rows (tap, ci), N = COUT, K = 16 voxels, both operands MN-major) into
 // the group's TMEM columns; at the end the four warps add their 128 lanes
 // (rows) of every group to dw with atomics.
@@ -301,10 +295,10 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant_
                 if (!ok) break;
                 uint8_t *a = smem + s * S::STAGE;
                 if (lane < ntap)
-                    load_tile<CIN / 8>(a + lane * (CIN / 8) * 2048, &xmap, &full[s], g, pos, tap % 3 - 1,
+                    load_tile(a + lane * (CIN / 8) * 2048, &xmap, &full[s], g, pos, tap % 3 - 1,
                                        (tap / 3) % 3 - 1, tap / 9 - 1);
                 else if (lane == 31)
-                    load_tile<COUT / 8>(a + S::A_BYTES, &gmap, &full[s], g, pos, 0, 0, 0);
+                    load_tile(a + S::A_BYTES, &gmap, &full[s], g, pos, 0, 0, 0);
                 __syncwarp();
             }
         }
@@ -503,7 +497,8 @@ gbsw_status conv_geometry(int NZ, int D, int H, int W, ConvGeom *g)
         bx = 32;
         by = 4;
     }
-    g->load = bx > 32 ? LOAD_VOXELS : bz > 1 && (D % bz == 0 || bz % D == 0) ? LOAD_SAMPLES : LOAD_ROWS;
+    g->load = bx > 32 ? LOAD_VOXELS : bz > 1 ? LOAD_SAMPLES : LOAD_ROWS;
+    g->sample_tiles = bz > 1 && bz % D == 0 ? 0 : ceil_div(D, bz);
     g->NZ = NZ;
     g->D = D;
     g->H = H;
@@ -513,7 +508,7 @@ gbsw_status conv_geometry(int NZ, int D, int H, int W, ConvGeom *g)
     g->box_z = bz;
     g->tiles_x = W / bx;
     g->tiles_y = H / by;
-    g->tiles_z = (NZ + bz - 1) / bz;
+    g->tiles_z = g->sample_tiles ? NZ / D * g->sample_tiles : ceil_div(NZ, bz);
     g->out_cg_total = g->out_cg0 = g->mask_cg_total = g->mask_cg0 = 0;
     return GBSW_OK;
 }
@@ -527,8 +522,7 @@ gbsw_status conv_tensor_map(const __nv_bfloat16 *base, const ConvGeom &g, int cg
     const cuuint64_t W = g.W, H = g.H, D = g.D, NZ = g.NZ, cg = cg_total;
     const cuuint64_t row = W * 16, group = H * row, plane = cg * group;  // bytes
     const cuuint32_t bx = g.box_x, by = g.box_y, bz = g.box_z;
-    // all channel groups at once, or (plane, group) by (plane, group)
-    const cuuint32_t bcg = bz > 1 && g.load != LOAD_SAMPLES ? 1u : (cuuint32_t)cg_total;
+    const cuuint32_t bcg = cg_total;  // all channel groups at once
     cuuint64_t dims[5], strides[4];
     cuuint32_t box[5];
     auto set = [&](int k, cuuint64_t dim, cuuint64_t stride, cuuint32_t b) {
@@ -552,7 +546,7 @@ gbsw_status conv_tensor_map(const __nv_bfloat16 *base, const ConvGeom &g, int cg
         set(4, 1, NZ * plane, 1);
         break;
     default: {
-        const cuuint32_t planes = std::min(g.D, g.box_z);
+        const cuuint32_t planes = g.sample_tiles ? g.box_z : g.D;  // more than the sample has: zero fill
         set(0, 8 * W, 0, 8 * bx);
         set(1, H, row, by);
         set(2, D, plane, planes);
