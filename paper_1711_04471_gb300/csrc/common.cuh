@@ -89,9 +89,10 @@ int sm_count();
 
 // Host-side fault injection for tests, from the GBSW_FAULT environment
 // variable (read at each call): "alloc" makes the create calls return
-// GBSW_ERR_OOM before any device allocation; "sync_timeout" gives the
-// ensemble kernel's grid barrier a zero spin budget, so that its bounded
-// wait gives up and the call reports GBSW_ERR_TIMEOUT.  No injection
+// GBSW_ERR_OOM before any device allocation; "sync_timeout" gives the waits
+// between thread blocks (the ensemble kernel's grid barrier, the exchanges of
+// sw_chip_kernel and sor_solve_kernel) no budget, so that they give up at
+// their first look and the call reports GBSW_ERR_TIMEOUT.  No injection
 // faults, traps or hangs a device.
 bool fault_injected(const char *what);
 

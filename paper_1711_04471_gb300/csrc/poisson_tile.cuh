@@ -62,7 +62,7 @@ constexpr int SORT_HALO = 4;                // halo groups that a thread of such
 constexpr int SORT_TILE_BYTES = 768;        // header of the dynamic shared memory
 constexpr int SORT_KINDS = 16;              // kinds of group by their diagonals
 constexpr int SORT_RB = 4;                  // rim items of a thread in flight
-constexpr long long SORT_WAIT_CYCLES = 4000000000LL;
+constexpr long long SORT_WAIT_CYCLES = 4000000000LL;  // budget of a wait: about 2 s
 
 // Words of SorTileArgs::sync.  The epoch (of the last half-sweep so far) goes
 // on from launch to launch of a register tile's solver; the others are 0 at launch.
@@ -80,6 +80,7 @@ struct SorTileRun {
     int chunk;        // predicted checks: iterations are counted in chunks (0: check every m)
     const double *s_in;   // fixed: stored stencil of p_hi for the first residual (NULL: form it)
     double *s_out;        // fixed: where the final residual stores the stencil (NULL: nowhere)
+    long long wait;       // clock budget of a wait for another CTA (filled in by launch_tiles)
 };
 
 struct SorTileArgs {
@@ -133,6 +134,7 @@ struct SorTile {
     int ncol, ps, e0;        // groups of one colour of e, its plane step, its group 0 of row (0, 0)
     int nrim, rim_half;      // rim rows; 16-byte words of one half of a published rim
     unsigned barriers, epoch;  // grid barriers passed; epoch of the last half-sweep so far
+    long long wait;          // clock budget of a wait for another CTA
     PoissonCtl c;
     double red[32];
 };
@@ -203,11 +205,11 @@ __device__ __forceinline__ int sort_row_of(int t, int ty, int tz)
 }
 
 // Waits until *p has reached `target` (the count only grows); false after the clock budget.
-__device__ __forceinline__ bool wait_reached(const unsigned *p, unsigned target)
+__device__ __forceinline__ bool wait_reached(const unsigned *p, unsigned target, long long budget)
 {
     const long long t0 = clock64();
     while ((int)(ld_relaxed_gpu(p) - target) < 0)
-        if (clock64() - t0 > SORT_WAIT_CYCLES) return false;
+        if (clock64() - t0 > budget) return false;
     return true;
 }
 
@@ -357,7 +359,7 @@ __device__ __noinline__ bool sort_grid_barrier()
         const unsigned n = ++T.barriers;
         fence_gpu();
         atomicAdd(T.A.sync + SORT_SYNC_COUNT, 1u);
-        late = !wait_reached(T.A.sync + SORT_SYNC_COUNT, n * gridDim.x);
+        late = !wait_reached(T.A.sync + SORT_SYNC_COUNT, n * gridDim.x, T.wait);
         fence_gpu();
     }
     return !__syncthreads_or(late);
@@ -400,13 +402,14 @@ __device__ __forceinline__ void sort_far_load(const uint4 *from, int half, SorFa
 }
 
 // Its values, once it carries the epoch (of the last half-sweep); *late if that does not come.
-__device__ __forceinline__ float4 sort_far_get(const uint4 *from, int half, unsigned epoch, SorFar &f, bool *late)
+__device__ __forceinline__ float4 sort_far_get(const uint4 *from, int half, unsigned epoch, SorFar &f, long long budget,
+                                               bool *late)
 {
     if (f.o < 0) return make_float4(0.f, 0.f, 0.f, 0.f);
     if (f.a.y != epoch || f.a.w != epoch || f.b.y != epoch || f.b.w != epoch) {
         const long long t0 = clock64();
         do {
-            if (clock64() - t0 > SORT_WAIT_CYCLES) {
+            if (clock64() - t0 > budget) {
                 *late = true;
                 break;
             }
@@ -879,7 +882,7 @@ __device__ __noinline__ bool sort_sweeps(int n_iter)
             }
         }
         if (!fetched) {
-            if (nb >= 0) late = !wait_reached(flag, target);
+            if (nb >= 0) late = !wait_reached(flag, target, T.wait);
             __syncwarp();
             look();
         }
@@ -964,8 +967,8 @@ __device__ __noinline__ bool sort_register_sweeps(int n_iter)
                     f1.o = hsrc[m + 1];
                     sort_far_load(from, half_words, f0);
                     sort_far_load(from, half_words, f1);
-                    if (f0.o >= 0) O[hdst[m]] = sort_far_get(from, half_words, epoch, f0, &late);
-                    if (f1.o >= 0) O[hdst[m + 1]] = sort_far_get(from, half_words, epoch, f1, &late);
+                    if (f0.o >= 0) O[hdst[m]] = sort_far_get(from, half_words, epoch, f0, T.wait, &late);
+                    if (f1.o >= 0) O[hdst[m + 1]] = sort_far_get(from, half_words, epoch, f1, T.wait, &late);
                 }
             }
         }
@@ -1082,6 +1085,7 @@ sor_solve_kernel(const __grid_constant__ SorTileArgs A, const __grid_constant__ 
         T.nrim = T.tz > 2 ? 2 * T.ty + (T.ty > 1 ? 2 : 1) * (T.tz - 2) : T.nrow;
         T.rim_half = A.rim_rows * P.G;
         T.barriers = 0;
+        T.wait = run.wait;
         T.epoch = A.sync[SORT_SYNC_EPOCH];
     }
     __syncthreads();

@@ -329,8 +329,9 @@ gbsw_status run_chip(gbsw_sw *s, int nsteps)
     if (nsteps == 0) return GBSW_OK;
     const int a = s->cur, b = 1 - a;
     unsigned epoch = s->epoch;
+    long long wait = fault_injected("sync_timeout") ? -1 : SWC_WAIT_CYCLES;
     const float *H = s->H, *ei = s->eta[a], *ui = s->u[a], *vi = s->v[a];
-    void *args[] = {&s->d, &s->chip, &nsteps, &epoch, &s->pub, &s->status, &H, &ei, &ui, &vi, &s->eta[b], &s->u[b], &s->v[b]};
+    void *args[] = {&s->d, &s->chip, &nsteps, &epoch, &wait, &s->pub, &s->status, &H, &ei, &ui, &vi, &s->eta[b], &s->u[b], &s->v[b]};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(s->chip.cx, s->chip.cy);
     cfg.blockDim = dim3(SWC_THREADS);

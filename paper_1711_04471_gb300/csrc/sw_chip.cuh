@@ -38,7 +38,7 @@ constexpr int SWC_MAX_T = 4;
 constexpr int SWC_GUARD = 2048;        // most columns of a region
 constexpr int SWC_ARRAYS = 6;          // shared FP32 arrays of a region
 constexpr int SWC_MAX_PER = 14;      // cells of a thread: with 15 and 16 the registers spill and the launches are faster
-constexpr long long SWC_WAIT_CYCLES = 4000000000LL;
+constexpr long long SWC_WAIT_CYCLES = 4000000000LL;  // budget of a wait: about 2 s
 
 // How a grid is cut: cx x cy tiles of tw x th cells (the last ones smaller),
 // T steps between exchanges, `per` cells per thread; cx = 0: it does not fit.
@@ -64,12 +64,13 @@ __device__ __forceinline__ void swc_store(uint4 *p, float a, float b, float c, u
 
 // nsteps steps from (eta_in, u_in, v_in) to (eta_out, u_out, v_out).  pub:
 // two arrays of ny x nx words (NULL with a single tile); epoch0: number of
-// the last exchange of earlier launches.  Cooperative launch: grid (cx, cy),
+// the last exchange of earlier launches; wait: clock budget of a wait for
+// another tile's word.  Cooperative launch: grid (cx, cy),
 // block SWC_THREADS, SWC_ARRAYS x PER x SWC_THREADS + 2 SWC_GUARD floats of
 // dynamic shared memory.
 template <int PER>
 __global__ void __launch_bounds__(SWC_THREADS, 1)
-sw_chip_kernel(SWDev p, SWChipPlan P, int nsteps, unsigned epoch0, uint4 *pub, int *status,
+sw_chip_kernel(SWDev p, SWChipPlan P, int nsteps, unsigned epoch0, long long wait, uint4 *pub, int *status,
                const float *__restrict__ H, const float *__restrict__ eta_in, const float *__restrict__ u_in,
                const float *__restrict__ v_in, float *__restrict__ eta_out, float *__restrict__ u_out,
                float *__restrict__ v_out)
@@ -199,7 +200,7 @@ sw_chip_kernel(SWDev p, SWChipPlan P, int nsteps, unsigned epoch0, uint4 *pub, i
                 if (v.w != epoch) {
                     const long long t0 = clock64();
                     do {
-                        if (clock64() - t0 > SWC_WAIT_CYCLES) {
+                        if (clock64() - t0 > wait) {
                             late = true;
                             break;
                         }

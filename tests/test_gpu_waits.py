@@ -1,0 +1,67 @@
+"""Waits between thread blocks that give up (GBSW_FAULT=sync_timeout gives them
+no budget): the kernels leave, the next synchronising call reports
+GBSW_ERR_TIMEOUT, and work without the injection then runs as before."""
+import numpy as np
+import pytest
+
+from paper_1711_04471_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+TIMEOUT = -6
+
+
+@pytest.fixture(scope="module")
+def N():
+    import paper_1711_04471_gb300 as P
+    P.build()
+    from paper_1711_04471_gb300 import _native
+    return _native
+
+
+def rhs(nx, ny, nz):
+    import torch
+    return torch.randn((nz, ny, nx), generator=torch.Generator(device="cuda").manual_seed(nx), device="cuda")
+
+
+def test_chip_steps_that_give_up_are_reported(N, monkeypatch):
+    from paper_1711_04471_gb300.sw import SW
+    inp = inputs.sw_hump(n=500)          # 147 tiles
+    with SW(inp.params(), inp.H, inp.eta0) as g:
+        g.set_tiling(3, 0)
+        g.step(100)
+        want = g.get_state()
+    monkeypatch.setenv("GBSW_FAULT", "sync_timeout")
+    for read in ("volume", "get_state"):
+        with SW(inp.params(), inp.H, inp.eta0) as g:
+            g.step(100)
+            with pytest.raises(N.GBSWError) as e:
+                getattr(g, read)()
+            assert e.value.status == TIMEOUT
+    monkeypatch.delenv("GBSW_FAULT")
+    with SW(inp.params(), inp.H, inp.eta0) as g:
+        g.step(100)
+        got = g.get_state()
+    for f in ("eta", "u", "v", "wet"):
+        assert np.array_equal(got[f], want[f]), f
+
+
+# the whole solve in one launch; checks as kernels of their own with the rows
+# in registers; and in shared memory (one row and plane per tile, so that a
+# tile looks at its neighbours' flags as soon as it has published its own)
+@pytest.mark.parametrize("shape", [(72, 48, 40), (256, 80, 96), (8192, 8, 4)])
+@pytest.mark.parametrize("kw", [dict(tol=1e-6, max_iter=200), dict(tol=-1.0, max_iter=20)])
+def test_solves_that_give_up_are_reported(N, monkeypatch, shape, kw):
+    import torch
+    from paper_1711_04471_gb300.les import poisson_solve
+    b = rhs(*shape)
+    first = torch.zeros_like(b)
+    s0 = poisson_solve(first, b, 4.0, **kw)
+    monkeypatch.setenv("GBSW_FAULT", "sync_timeout")
+    with pytest.raises(N.GBSWError) as e:
+        poisson_solve(torch.zeros_like(b), b, 4.0, **kw)
+    assert e.value.status == TIMEOUT
+    monkeypatch.delenv("GBSW_FAULT")
+    again = torch.zeros_like(b)
+    assert poisson_solve(again, b, 4.0, **kw) == s0
+    assert torch.equal(again, first)
