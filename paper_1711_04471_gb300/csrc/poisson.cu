@@ -514,7 +514,7 @@ gbsw_status PoissonSolver::launch_tiles(const SorTileRun &run, cudaStream_t stre
     A.ctl = ctl;
     const int nblocks = plan_.py * plan_.pz;
     // register tiles: the epoch goes on; others: it starts at 0 with the tiles' flags
-    const int w0 = plan_.items ? SORT_SYNC_COUNT : 0, words = plan_.items ? 1 : 32 * (nblocks + 1);
+    const int w0 = plan_.items ? SORT_SYNC_COUNT : 0, words = plan_.items ? 2 : 32 * (nblocks + 1);
     GBSW_CUDA_TRY(cudaMemsetAsync(sync_ + w0, 0, (size_t)words * sizeof(unsigned), stream));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nblocks);

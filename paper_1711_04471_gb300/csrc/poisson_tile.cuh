@@ -68,6 +68,7 @@ constexpr long long SORT_WAIT_CYCLES = 4000000000LL;  // budget of a wait: about
 // on from launch to launch of a register tile's solver; the others are 0 at launch.
 constexpr int SORT_SYNC_EPOCH = 0;
 constexpr int SORT_SYNC_COUNT = 1;    // CTAs that have come to a grid barrier
+constexpr int SORT_SYNC_LATE = 2;     // a CTA has given up a wait
 
 // How a solve ends and where its checks come.
 struct SorTileRun {
@@ -1133,7 +1134,7 @@ sor_solve_kernel(const __grid_constant__ SorTileArgs A, const __grid_constant__ 
         if (tid == 0) {
             if (!ok) {
                 atomicCAS(&A.ctl->status, DEV_OK, DEV_TIMEOUT);
-                atomicAdd(A.sync + SORT_SYNC_EPOCH, 1u << 24);
+                if (atomicExch(A.sync + SORT_SYNC_LATE, 1u) == 0) atomicAdd(A.sync + SORT_SYNC_EPOCH, 1u << 24);
             } else if (blockIdx.x == 0) {
                 A.ctl->since = n;
                 if (I > 0) atomicAdd(A.sync + SORT_SYNC_EPOCH, 2u * n);
@@ -1185,12 +1186,21 @@ sor_solve_kernel(const __grid_constant__ SorTileArgs A, const __grid_constant__ 
         }
         if (ok) sort_write_tile();
         if (tid == 0) {
+            // One CTA may pass the last barrier while another gives it up, its
+            // part of p not written: the solve has then failed, whichever of the
+            // two comes here first.  The one raises the flag, then the status;
+            // the other writes its status, then looks at the flag.
             if (!ok) {
-                atomicCAS(&A.ctl->status, DEV_OK, DEV_TIMEOUT);
-                atomicAdd(A.sync + SORT_SYNC_EPOCH, 1u << 24);  // past every epoch that this solve may have published
+                const bool first_late = atomicExch(A.sync + SORT_SYNC_LATE, 1u) == 0;
+                __threadfence();
+                atomicExch(&A.ctl->status, DEV_TIMEOUT);
+                // past every epoch that this solve may have published
+                if (first_late) atomicAdd(A.sync + SORT_SYNC_EPOCH, 1u << 24);
             } else if (blockIdx.x == 0) {
                 *A.ctl = T.c;
                 A.sync[SORT_SYNC_EPOCH] = T.epoch;
+                __threadfence();
+                if (ld_relaxed_gpu(A.sync + SORT_SYNC_LATE)) atomicExch(&A.ctl->status, DEV_TIMEOUT);
             }
         }
     }

@@ -65,3 +65,21 @@ def test_solves_that_give_up_are_reported(N, monkeypatch, shape, kw):
     again = torch.zeros_like(b)
     assert poisson_solve(again, b, 4.0, **kw) == s0
     assert torch.equal(again, first)
+
+
+def test_a_finished_tile_does_not_hide_anothers_timeout(N, monkeypatch):
+    """A right-hand side whose square sum is below 1e-60 is solved by the first
+    check, so the last block to come to its barrier finishes while the others
+    give up.  Subnormal values, which take longer, make that the first block,
+    the one that writes the solve's result: the report must not depend on it."""
+    import torch
+    from paper_1711_04471_gb300.les import poisson_solve
+    b = torch.zeros((96, 96, 128))
+    b[:8, :8] = 1e-40           # the first of 12 x 12 tiles
+    b = b.cuda()
+    p = torch.zeros_like(b)
+    monkeypatch.setenv("GBSW_FAULT", "sync_timeout")
+    for _ in range(1000):
+        with pytest.raises(N.GBSWError) as e:
+            poisson_solve(p, b, 4.0)
+        assert e.value.status == TIMEOUT
