@@ -150,8 +150,10 @@ gbsw_status sw_create(const gbsw_sw_params *params, const double *H, const doubl
  * context stream; several steps are fused per kernel launch.  With the
  * automatic tiling a grid that fits in the SMs' registers and shared memory
  * takes all steps of the call in one cooperative launch (not while the
- * stream is being captured); its bounded waits between SMs report
- * GBSW_ERR_TIMEOUT at the next sw_volume or sw_get_state. */
+ * stream is being captured).  If one of its bounded waits between SMs gives
+ * up, the state is torn: the next sw_volume, sw_get_state or sw_autotune
+ * reports GBSW_ERR_TIMEOUT, and so do all calls of these and sw_step from
+ * then on, until sw_set_state has replaced eta, u and v. */
 gbsw_status sw_step(gbsw_sw *sw, int nsteps);
 
 /*
@@ -172,7 +174,8 @@ gbsw_status sw_get_state(gbsw_sw *sw, float *eta, float *u, float *v, uint8_t *w
 
 /* Replace the state from host buffers in the layout of sw_get_state (wall
  * faces are ignored and kept 0).  Any of eta, u, v may be NULL to keep the
- * current field.  Synchronous. */
+ * current field.  With all three given a context that reported
+ * GBSW_ERR_TIMEOUT is usable again.  Synchronous. */
 gbsw_status sw_set_state(gbsw_sw *sw, const float *eta, const float *u, const float *v);
 
 /* Number of time steps fused per kernel launch (temporal blocking depth):

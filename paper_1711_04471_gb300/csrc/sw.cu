@@ -107,6 +107,7 @@ struct gbsw_sw {
     int *status;            // device status word of the chip kernel
     int *h_status;          // pinned copy
     bool status_due;        // a chip launch has been enqueued since the status was last read
+    gbsw_status failed;     // a chip launch gave up a wait: the state is torn until sw_set_state replaces all of it
 };
 
 namespace {
@@ -359,11 +360,20 @@ gbsw_status status_read(gbsw_sw *s)
 
 gbsw_status status_judge(gbsw_sw *s)
 {
-    if (!s->status_due) return GBSW_OK;
+    if (s->status_due) {
+        s->status_due = false;
+        s->failed = dev_status_to_gbsw(*s->h_status);
+    }
+    return s->failed;
+}
+
+// The state is whole again: whatever earlier launches report no longer counts.
+gbsw_status status_clear(gbsw_sw *s)
+{
+    GBSW_CUDA_TRY(cudaMemsetAsync(s->status, 0, sizeof(int), s->stream));
     s->status_due = false;
-    const gbsw_status st = dev_status_to_gbsw(*s->h_status);
-    if (st != GBSW_OK) cudaMemsetAsync(s->status, 0, sizeof(int), s->stream);
-    return st;
+    s->failed = GBSW_OK;
+    return GBSW_OK;
 }
 
 // True if the context's stream is being captured: the chip kernel's exchange
@@ -580,6 +590,7 @@ gbsw_status sw_step(gbsw_sw *s, int nsteps)
 {
     gbsw::NvtxRange nvtx_range("sw_step");
     if (!s || nsteps < 0) return GBSW_ERR_ARG;
+    if (s->failed != GBSW_OK) return s->failed;
     if (s->blocking == 0 && s->rows == 0 && s->chip.cx && !capturing(s)) return run_chip(s, nsteps);
     const int T = tiling_T(s);
     return run_steps(s, nsteps, T, tiling_rows(s, T));
@@ -589,6 +600,12 @@ gbsw_status sw_autotune(gbsw_sw *s, int trial_steps, int *T_out, int *rows_out)
 {
     gbsw::NvtxRange nvtx_range("sw_autotune");
     if (!s || trial_steps < 1 || trial_steps > 100000) return GBSW_ERR_ARG;
+    if (s->status_due) {  // a state that is torn already is not worth a tiling
+        const gbsw_status due = status_read(s);
+        if (due != GBSW_OK) return due;
+        GBSW_CUDA_TRY(cudaStreamSynchronize(s->stream));
+    }
+    if (status_judge(s) != GBSW_OK) return s->failed;
     const size_t fb = (size_t)s->d.pitch * (size_t)s->d.ny * sizeof(float);
     float *save[3] = {nullptr, nullptr, nullptr};
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -657,7 +674,12 @@ gbsw_status sw_autotune(gbsw_sw *s, int trial_steps, int *T_out, int *rows_out)
             if (st == GBSW_OK &&
                 (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
                 st = GBSW_ERR_CUDA;
-            automatic = st == GBSW_OK && ms / trial_steps < best;
+            if (st == GBSW_OK && (st = status_read(s)) == GBSW_OK && cudaStreamSynchronize(s->stream) != cudaSuccess)
+                st = GBSW_ERR_CUDA;
+            // a trial that gave up a wait is not a choice, and leaves nothing to report: the state is restored below
+            automatic = st == GBSW_OK && *s->h_status == DEV_OK && ms / trial_steps < best;
+            const gbsw_status cleared = status_clear(s);
+            if (st == GBSW_OK) st = cleared;
         }
         // restore the state: results do not depend on the tiling, so the
         // trials leave no trace
@@ -748,6 +770,10 @@ gbsw_status sw_set_state(gbsw_sw *s, const float *eta, const float *u, const flo
     if (v) {
         GBSW_CUDA_TRY(cudaMemcpy2DAsync(s->v[c], dp, v + nx, row, row, ny, cudaMemcpyHostToDevice, s->stream));
         GBSW_CUDA_TRY(cudaMemsetAsync(s->v[c] + (size_t)(ny - 1) * s->d.pitch, 0, row, s->stream));
+    }
+    if (eta && u && v) {
+        const gbsw_status st = status_clear(s);
+        if (st != GBSW_OK) return st;
     }
     GBSW_CUDA_TRY(cudaStreamSynchronize(s->stream));
     return GBSW_OK;

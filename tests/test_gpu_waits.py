@@ -83,3 +83,58 @@ def test_a_finished_tile_does_not_hide_anothers_timeout(N, monkeypatch):
         with pytest.raises(N.GBSWError) as e:
             poisson_solve(p, b, 4.0)
         assert e.value.status == TIMEOUT
+
+
+def test_a_torn_state_stays_reported_until_it_is_replaced(N, monkeypatch):
+    from paper_1711_04471_gb300.sw import SW
+    inp = inputs.sw_hump(n=500)
+    with SW(inp.params(), inp.H, inp.eta0) as g:
+        g.step(7)
+        start = g.get_state()
+        g.step(100)
+        want, vol = g.get_state(), g.volume()
+
+    def refused(call):
+        with pytest.raises(N.GBSWError) as e:
+            call()
+        assert e.value.status == TIMEOUT
+
+    with SW(inp.params(), inp.H, inp.eta0) as g:
+        monkeypatch.setenv("GBSW_FAULT", "sync_timeout")
+        g.step(100)
+        refused(g.volume)
+        monkeypatch.delenv("GBSW_FAULT")
+        for call in (g.get_state, g.volume, lambda: g.step(1), lambda: g.autotune(10), g.get_state):
+            refused(call)
+        g.set_state(eta=start["eta"], u=start["u"])     # v is still torn
+        refused(g.volume)
+        g.set_state(eta=start["eta"], u=start["u"], v=start["v"])
+        g.step(100)
+        got = g.get_state()
+        assert g.volume() == vol
+        # a timeout that nobody has asked about yet does not outlive the state it tore
+        monkeypatch.setenv("GBSW_FAULT", "sync_timeout")
+        g.step(100)
+        monkeypatch.delenv("GBSW_FAULT")
+        g.set_state(eta=start["eta"], u=start["u"], v=start["v"])
+        g.step(100)
+        again = g.get_state()
+        assert g.volume() == vol
+    for f in ("eta", "u", "v", "wet"):
+        assert np.array_equal(got[f], want[f]), f
+        assert np.array_equal(again[f], want[f]), f
+
+
+def test_autotune_does_not_keep_or_report_a_trial_that_gave_up(N, monkeypatch):
+    from paper_1711_04471_gb300.sw import SW
+    inp = inputs.sw_hump(n=500)
+    with SW(inp.params(), inp.H, inp.eta0) as a, SW(inp.params(), inp.H, inp.eta0) as b:
+        a.step(100)
+        want, vol = a.get_state(), a.volume()
+        monkeypatch.setenv("GBSW_FAULT", "sync_timeout")
+        b.autotune(trial_steps=12)
+        b.step(100)                  # launches: they have no waits
+        got = b.get_state()
+        assert b.volume() == vol
+    for f in ("eta", "u", "v", "wet"):
+        assert np.array_equal(got[f], want[f]), f
