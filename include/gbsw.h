@@ -370,7 +370,10 @@ gbsw_status les_create(const gbsw_les_params *params, const uint8_t *solid, void
 /*
  * Advance nsteps steps.  stats: host array of nsteps records or NULL.
  * Synchronises at the end; returns the worst per-step status
- * (GBSW_NOT_CONVERGED if any solve stopped at max_iter).
+ * (GBSW_NOT_CONVERGED if any solve stopped at max_iter).  After
+ * GBSW_ERR_TIMEOUT (a bounded wait inside a pressure solve gave up) the
+ * pressure is that of an unfinished solve, and later steps start from it:
+ * go back to a state taken before.
  */
 gbsw_status les_step(gbsw_les *les, int nsteps, gbsw_les_stats *stats);
 

@@ -756,7 +756,7 @@ gbsw_status PoissonSolver::build_graph_tiles()
     if (err == cudaSuccess) {
         chk(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
         if (err == cudaSuccess) {
-            st = launch_tiles(SorTileRun{0, predict ? -1 : m, 0.0, 0.0, 0, 0, predict ? chunk() : 0, nullptr, nullptr, 0}, cs);
+            st = launch_tiles(SorTileRun{0, predict ? -1 : m, 0.0, 0.0, 0, 0, predict ? chunk() : 0, nullptr, nullptr, nullptr, 0}, cs);
             poisson_resid_kernel<false><<<rgrid, POI_RED_THREADS, 0, cs>>>(d, b, p_hi, r[0], r[1], partials, nullptr,
                                                                            nullptr, nullptr);
             poisson_test_kernel<true><<<1, POI_RED_THREADS, 0, cs>>>(partials, rblocks, ctl, tol, max_iter, m, 1, predict,
@@ -900,7 +900,7 @@ gbsw_status PoissonSolver::enqueue()
     s_valid_ = false;  // the folds change p_hi and no stencil is stored
     if (plan_.psm)
         return launch_tiles(SorTileRun{0, 0, tol, tol * tol * (1.0 + 1e-12), max_iter, m, predict_ ? chunk() : 0, nullptr,
-                                       nullptr, 0}, stream);
+                                       nullptr, nullptr, 0}, stream);
     if (dirty_) {
         gbsw_status st = build_graph();
         if (st != GBSW_OK) return st;
@@ -921,8 +921,8 @@ gbsw_status PoissonSolver::enqueue_fixed(int niter, bool use_graph)
     if (plan_.psm) {
         const double *s_in = s_valid_ ? s_cache : nullptr;
         s_valid_ = false;
-        const gbsw_status st = launch_tiles(SorTileRun{1, niter, 0.0, 0.0, niter, niter, 0, s_in, s_cache, 0}, stream);
-        s_valid_ = st == GBSW_OK;
+        const gbsw_status st = launch_tiles(SorTileRun{1, niter, 0.0, 0.0, niter, niter, 0, s_in, s_cache, s_ok, 0}, stream);
+        s_valid_ = st == GBSW_OK;  // and the kernel's own word s_ok says whether the solve came to its end
         return st;
     }
     // the first residual may reuse the last fixed-count solve's stencil only
@@ -975,7 +975,7 @@ gbsw_status PoissonSolver::record_fixed(int niter, cudaStream_t stream)
                                                                       nullptr);
     poisson_test_kernel<false><<<1, POI_RED_THREADS, 0, stream>>>(partials, rblocks, ctl, 0.0, niter, 0, 0, 0, 0);
     if (plan_.py) {
-        const gbsw_status st = launch_tiles(SorTileRun{0, niter, 0.0, 0.0, 0, 0, 0, nullptr, nullptr, 0}, stream);
+        const gbsw_status st = launch_tiles(SorTileRun{0, niter, 0.0, 0.0, 0, 0, 0, nullptr, nullptr, nullptr, 0}, stream);
         if (st != GBSW_OK) return st;
     } else {
         cudaError_t err = launch_iterations(d, niter, om, h2, e, r, stream);

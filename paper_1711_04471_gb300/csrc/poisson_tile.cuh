@@ -79,8 +79,9 @@ struct SorTileRun {
     int max_iter;
     int m;            // check interval
     int chunk;        // predicted checks: iterations are counted in chunks (0: check every m)
-    const double *s_in;   // fixed: stored stencil of p_hi for the first residual (NULL: form it)
+    const double *s_in;   // fixed: stored stencil of p_hi for the first residual if *s_ok (NULL: form it)
     double *s_out;        // fixed: where the final residual stores the stencil (NULL: nowhere)
+    int *s_ok;            // fixed: 1 if the stencil is that of p_hi; 0 after a solve that gave up a wait
     long long wait;       // clock budget of a wait for another CTA (filled in by launch_tiles)
 };
 
@@ -136,6 +137,7 @@ struct SorTile {
     int nrim, rim_half;      // rim rows; 16-byte words of one half of a published rim
     unsigned barriers, epoch;  // grid barriers passed; epoch of the last half-sweep so far
     long long wait;          // clock budget of a wait for another CTA
+    bool stored;             // the stored stencil is that of p_hi
     PoissonCtl c;
     double red[32];
 };
@@ -1087,6 +1089,7 @@ sor_solve_kernel(const __grid_constant__ SorTileArgs A, const __grid_constant__ 
         T.rim_half = A.rim_rows * P.G;
         T.barriers = 0;
         T.wait = run.wait;
+        T.stored = run.s_in && *run.s_ok != 0;
         T.epoch = A.sync[SORT_SYNC_EPOCH];
     }
     __syncthreads();
@@ -1147,7 +1150,7 @@ sor_solve_kernel(const __grid_constant__ SorTileArgs A, const __grid_constant__ 
         int ran = 0;
         sort_read_tile();
         for (;;) {
-            sort_residual(first ? run.s_in : nullptr, !first && run.fixed ? run.s_out : nullptr, first);
+            sort_residual(first && T.stored ? run.s_in : nullptr, !first && run.fixed ? run.s_out : nullptr, first);
             ok = sort_grid_barrier();
             if (!ok) break;
             if (tid < 32) {
@@ -1189,18 +1192,23 @@ sor_solve_kernel(const __grid_constant__ SorTileArgs A, const __grid_constant__ 
             // One CTA may pass the last barrier while another gives it up, its
             // part of p not written: the solve has then failed, whichever of the
             // two comes here first.  The one raises the flag, then the status;
-            // the other writes its status, then looks at the flag.
+            // the other writes its status, then looks at the flag.  (s_ok too.)
             if (!ok) {
                 const bool first_late = atomicExch(A.sync + SORT_SYNC_LATE, 1u) == 0;
                 __threadfence();
                 atomicExch(&A.ctl->status, DEV_TIMEOUT);
+                if (run.s_out) atomicExch(run.s_ok, 0);
                 // past every epoch that this solve may have published
                 if (first_late) atomicAdd(A.sync + SORT_SYNC_EPOCH, 1u << 24);
             } else if (blockIdx.x == 0) {
                 *A.ctl = T.c;
                 A.sync[SORT_SYNC_EPOCH] = T.epoch;
+                if (run.s_out) *run.s_ok = 1;
                 __threadfence();
-                if (ld_relaxed_gpu(A.sync + SORT_SYNC_LATE)) atomicExch(&A.ctl->status, DEV_TIMEOUT);
+                if (ld_relaxed_gpu(A.sync + SORT_SYNC_LATE)) {
+                    atomicExch(&A.ctl->status, DEV_TIMEOUT);
+                    if (run.s_out) atomicExch(run.s_ok, 0);
+                }
             }
         }
     }

@@ -138,3 +138,28 @@ def test_autotune_does_not_keep_or_report_a_trial_that_gave_up(N, monkeypatch):
         assert b.volume() == vol
     for f in ("eta", "u", "v", "wet"):
         assert np.array_equal(got[f], want[f]), f
+
+
+def test_a_fixed_solve_that_gave_up_leaves_no_stencil(N, monkeypatch):
+    """The final residual of a fixed-count solve stores the stencil of p for
+    the next solve's first one.  After a solve that gave up, the next forms it
+    anew: a context whose p is written back (which drops the stencil) and one
+    whose p is left alone go on alike."""
+    from paper_1711_04471_gb300.les import LES
+    p0 = np.random.default_rng(3).standard_normal((42, 50, 74))
+    out = []
+    for write_back in (True, False):
+        with LES(72, 48, 40) as les:
+            les.set_fixed_iterations(20)
+            les.set("p", p0)
+            monkeypatch.setenv("GBSW_FAULT", "sync_timeout")
+            with pytest.raises(N.GBSWError) as e:
+                les.step(1)
+            assert e.value.status == TIMEOUT
+            monkeypatch.delenv("GBSW_FAULT")
+            if write_back:
+                les.set("p", les.get("p"))
+            les.step(2)
+            out.append([les.get(f) for f in ("p", "u", "v", "w")])
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
