@@ -92,7 +92,9 @@ int sm_count();
 // GBSW_ERR_OOM before any device allocation; "sync_timeout" gives the waits
 // between thread blocks (the ensemble kernel's grid barrier, the exchanges of
 // sw_chip_kernel and sor_solve_kernel) no budget, so that they give up at
-// their first look and the call reports GBSW_ERR_TIMEOUT.  No injection
+// their first look and the call reports GBSW_ERR_TIMEOUT; "occupancy" makes
+// the create and solve calls find no room for the cooperative kernels, so
+// that the launch-by-launch paths run.  No injection
 // faults, traps or hangs a device.
 bool fault_injected(const char *what);
 

@@ -484,9 +484,9 @@ static SorTilePlan sort_plan(int nx, int ny, int nz)
     int per_sm = 0;
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, best.threads, best.smem) != cudaSuccess ||
-        per_sm < 1) {
+        per_sm < 1 || fault_injected("occupancy")) {
         cudaGetLastError();
-        best.py = 0;
+        return SorTilePlan{};  // nothing of the plan stays: each of py, items and psm selects a path
     }
     return best;
 }

@@ -317,9 +317,9 @@ SWChipPlan chip_plan(int nx, int ny)
     int per_sm = 0;
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chip_smem(best.per)) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, SWC_THREADS, chip_smem(best.per)) != cudaSuccess ||
-        per_sm < 1) {
+        per_sm < 1 || fault_injected("occupancy")) {
         cudaGetLastError();
-        best.cx = 0;
+        return SWChipPlan{};
     }
     return best;
 }

@@ -163,3 +163,33 @@ def test_a_fixed_solve_that_gave_up_leaves_no_stencil(N, monkeypatch):
             out.append([les.get(f) for f in ("p", "u", "v", "w")])
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("shape", [(72, 48, 40), (256, 80, 96), (8192, 8, 4)])
+def test_solves_without_room_for_the_cooperative_kernel(N, monkeypatch, shape):
+    """The half-sweep launches take over, with the same iterates; the residual
+    norms are FP64 sums in another order."""
+    import torch
+    from paper_1711_04471_gb300.les import poisson_solve
+    b = rhs(*shape)
+    for kw in (dict(tol=1e-6, max_iter=200), dict(tol=-1.0, max_iter=21)):
+        p, q = torch.zeros_like(b), torch.zeros_like(b)
+        want = poisson_solve(p, b, 4.0, **kw)
+        monkeypatch.setenv("GBSW_FAULT", "occupancy")
+        got = poisson_solve(q, b, 4.0, **kw)
+        monkeypatch.delenv("GBSW_FAULT")
+        assert got[:2] == want[:2] and abs(got[2] - want[2]) <= 1e-12 * want[2]
+        assert torch.equal(p, q)
+
+
+def test_steps_without_room_for_the_cooperative_kernel(N, monkeypatch):
+    from paper_1711_04471_gb300.sw import SW
+    inp = inputs.sw_hump(n=300)
+    out = []
+    for fault in ("", "occupancy"):
+        monkeypatch.setenv("GBSW_FAULT", fault)
+        with SW(inp.params(), inp.H, inp.eta0) as g:
+            g.step(50)
+            out.append(g.get_state())
+    for f in ("eta", "u", "v", "wet"):
+        assert np.array_equal(out[0][f], out[1][f]), f
