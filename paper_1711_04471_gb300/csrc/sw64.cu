@@ -142,14 +142,23 @@ __device__ __forceinline__ void s64_wait()
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// Launch of the kernels that set up and read the state: columns x rows, a
+// block taking rows y, y + gridDim.y, ... (a grid has at most 65535 in y).
+dim3 s64_rows_grid(int columns, int rows)
+{
+    return dim3(gbsw::ceil_div(columns, S64_THREADS), std::min(rows, 65535));
+}
+
 // h = H + eta on the interior (the initial state).
 __global__ void __launch_bounds__(S64_THREADS)
 sw64_depth_kernel(S64Dev p, const double *H, const double *eta, double *h)
 {
-    const int i = blockIdx.x * S64_THREADS + threadIdx.x + 1, j = blockIdx.y + 1;
+    const int i = blockIdx.x * S64_THREADS + threadIdx.x + 1;
     if (i > p.nx) return;
-    const long long c = (long long)j * p.pitch + i;
-    h[c] = __dadd_rn(H[c], eta[c]);
+    for (int j = blockIdx.y + 1; j <= p.ny; j += gridDim.y) {
+        const long long c = (long long)j * p.pitch + i;
+        h[c] = __dadd_rn(H[c], eta[c]);
+    }
 }
 
 // Map 1 ("dyn", momentum): u' and its flux on the east faces i = 1 .. nx-1,
@@ -224,18 +233,21 @@ sw64_shapiro_kernel(S64Dev p, const double *H, const double *h, const double *es
 
 // Rows 0 .. rows-1 of `width` elements from `src` (row pitch p.pitch) packed into dst.
 __global__ void __launch_bounds__(S64_THREADS)
-sw64_pack_kernel(S64Dev p, const double *src, int width, double *dst)
+sw64_pack_kernel(S64Dev p, const double *src, int width, int rows, double *dst)
 {
-    const int i = blockIdx.x * S64_THREADS + threadIdx.x, j = blockIdx.y;
-    if (i < width) dst[(size_t)j * width + i] = src[(size_t)j * p.pitch + i];
+    const int i = blockIdx.x * S64_THREADS + threadIdx.x;
+    if (i >= width) return;
+    for (int j = blockIdx.y; j < rows; j += gridDim.y) dst[(size_t)j * width + i] = src[(size_t)j * p.pitch + i];
 }
 
 // Wet mask of the state as bytes.
 __global__ void __launch_bounds__(S64_THREADS)
 sw64_wet_kernel(S64Dev p, const double *h, uint8_t *wet)
 {
-    const int i = blockIdx.x * S64_THREADS + threadIdx.x, j = blockIdx.y;
-    if (i < p.nx) wet[(size_t)j * p.nx + i] = h[(size_t)(j + 1) * p.pitch + i + 1] > p.hmin;
+    const int i = blockIdx.x * S64_THREADS + threadIdx.x;
+    if (i >= p.nx) return;
+    for (int j = blockIdx.y; j < p.ny; j += gridDim.y)
+        wet[(size_t)j * p.nx + i] = h[(size_t)(j + 1) * p.pitch + i + 1] > p.hmin;
 }
 
 // FP64 volume partials over rows b, b + S64_VOL_BLOCKS, ... (fixed order).
@@ -418,8 +430,7 @@ gbsw_status sw64_create(const gbsw_sw_params *params, const double *H, const dou
     if (err == cudaSuccess)
         err = cudaMemcpy2DAsync(s->eta + s->pitch + 1, dp, e.data(), hp, hp, P.ny, cudaMemcpyHostToDevice, s->stream);
     if (err == cudaSuccess) {
-        const dim3 g(ceil_div(P.nx, S64_THREADS), P.ny);
-        sw64_depth_kernel<<<g, S64_THREADS, 0, s->stream>>>(s64_dev(s), s->H, s->eta, s->h[0]);
+        sw64_depth_kernel<<<s64_rows_grid(P.nx, P.ny), S64_THREADS, 0, s->stream>>>(s64_dev(s), s->H, s->eta, s->h[0]);
         err = cudaGetLastError();
     }
     if (err == cudaSuccess) err = cudaStreamSynchronize(s->stream);
@@ -477,8 +488,7 @@ gbsw_status sw64_get_state(gbsw_sw64 *s, double *eta, double *u, double *v, uint
     // row by row.
     const S64Dev d = s64_dev(s);
     auto copy = [&](double *dst, const double *src, int width, int rows) -> gbsw_status {
-        const dim3 g(ceil_div(width, S64_THREADS), rows);
-        sw64_pack_kernel<<<g, S64_THREADS, 0, s->stream>>>(d, src, width, s->es);
+        sw64_pack_kernel<<<s64_rows_grid(width, rows), S64_THREADS, 0, s->stream>>>(d, src, width, rows, s->es);
         GBSW_LAUNCH_CHECK();
         GBSW_CUDA_TRY(cudaMemcpyAsync(dst, s->es, (size_t)width * rows * sizeof(double), cudaMemcpyDeviceToHost,
                                       s->stream));
@@ -490,8 +500,7 @@ gbsw_status sw64_get_state(gbsw_sw64 *s, double *eta, double *u, double *v, uint
     if (v && st == GBSW_OK) st = copy(v, s->v + 1, nx, ny + 1);         // north faces j = 0..ny of columns 1..nx
     if (st != GBSW_OK) return st;
     if (wet) {
-        const dim3 g(ceil_div(nx, S64_THREADS), ny);
-        sw64_wet_kernel<<<g, S64_THREADS, 0, s->stream>>>(d, s->h[s->cur], (uint8_t *)s->es);
+        sw64_wet_kernel<<<s64_rows_grid(nx, ny), S64_THREADS, 0, s->stream>>>(d, s->h[s->cur], (uint8_t *)s->es);
         GBSW_LAUNCH_CHECK();
         GBSW_CUDA_TRY(cudaMemcpyAsync(wet, s->es, (size_t)nx * ny, cudaMemcpyDeviceToHost, s->stream));
     }
