@@ -456,9 +456,10 @@ gbsw_status sw64_step(gbsw_sw64 *s, int nsteps)
     }
     for (int k = 0; k < left && e == cudaSuccess; ++k) {
         e = s64_enqueue(s, d, s->cur, s->stream, k > 0);
-        s->cur = 1 - s->cur;
+        if (e == cudaSuccess) s->cur = 1 - s->cur;
     }
     if (e != cudaSuccess) {
+        cudaGetLastError();  // reported here, not by the next call
         record_cuda_error(e, "sw64_step", __FILE__, __LINE__);
         return GBSW_ERR_CUDA;
     }

@@ -32,3 +32,20 @@ def test_tall_grids_are_set_up_and_read(SW64, ny):
     assert st["u"].shape == (ny, 4) and not st["u"].any()
     assert st["v"].shape == (ny + 1, 3) and not st["v"].any()
     assert vol == pytest.approx(100.0 * (H + eta).sum(), rel=1e-13)
+
+
+@pytest.mark.parametrize("steps", [1, 16])
+def test_a_step_that_cannot_be_launched_leaves_the_state(SW64, steps):
+    """A step has a block row per grid row, so 70000 rows cannot be launched:
+    the call fails, and the state reads as before it."""
+    from paper_1711_04471_gb300._native import GBSWError
+    rng = np.random.default_rng(1)
+    H = rng.uniform(-1.0, 10.0, (70000, 3))
+    with SW64(dict(nx=3, ny=70000, dx=10.0, dy=10.0, dt=0.1), H, np.maximum(0.0, -H)) as g:
+        before = g.get_state()
+        with pytest.raises(GBSWError) as e:
+            g.step(steps)
+        assert e.value.status == -2
+        after = g.get_state()
+    for f in ("eta", "u", "v", "wet"):
+        assert np.array_equal(before[f], after[f]), f
