@@ -661,7 +661,7 @@ def run_sw_paper(args, rank, world, local):
 
     import paper_1711_04471_gb300 as P
     from paper_1711_04471_gb300 import inputs
-    from paper_1711_04471_gb300.sw import SW
+    from paper_1711_04471_gb300.sw import ONE_LAUNCH, SW
     P.build()
     torch.cuda.set_device(local)
     res = []
@@ -685,9 +685,11 @@ def run_sw_paper(args, rank, world, local):
                 oracle.use_openmp(False)
             cpu["threads"] = oracle.threads()
         res.append({"n": n, "seconds_10000_steps": t, "cell_updates_per_s": n * n * 10000 / t,
-                    "tiling": {"steps_per_launch": tiling[0], "rows_per_block": tiling[1],
+                    "tiling": {"steps_per_launch": 10000 if tiling[1] == ONE_LAUNCH else tiling[0],
+                               "rows_per_block": None if tiling[1] == ONE_LAUNCH else tiling[1],
                                "kernel": ("tile, %d rows per tile" % (32 if tiling[1] == -1 else -tiling[1])
-                                          if tiling[1] < 0 else "streaming")},
+                                          if tiling[1] < 0 else "on the chip, one launch per call"
+                                          if tiling[1] == ONE_LAUNCH else "streaming")},
                     "oracle_cell_updates_per_s_1thread": cpu.get(False),
                     "oracle_cell_updates_per_s_all_cores": cpu.get(True), "oracle_threads": cpu.get("threads")})
     if rank != 0:

@@ -190,8 +190,11 @@ gbsw_status sw_set_blocking(gbsw_sw *sw, int steps_per_launch);
  * holds 32 columns x h rows and a 2T-cell halo in shared memory, with
  * h = 32 for rows = -1 and h = -rows for rows <= -2 (T = 1..3 given
  * explicitly; h at most 52, 43, 34 for T = 1, 2, 3, else GBSW_ERR_ARG).
+ * rows = GBSW_SW_ONE_LAUNCH, as sw_autotune reports it, is the automatic
+ * setting with its one-launch path where the grid fits (else one segment).
  * Results do not depend on the tiling (every operation is rounded as
  * written). */
+#define GBSW_SW_ONE_LAUNCH (1 << 30)
 gbsw_status sw_set_tiling(gbsw_sw *sw, int steps_per_launch, int rows);
 
 /* Choose the tiling by measurement: times trial_steps (1..100000, rounded
@@ -202,11 +205,16 @@ gbsw_status sw_set_tiling(gbsw_sw *sw, int steps_per_launch, int rows);
  * keeps the fastest (written to *T_out, *rows_out in the encoding of
  * sw_set_tiling, if non-NULL) and restores the state exactly.  The automatic
  * setting's one-launch path is timed too and kept if it is faster than all
- * of these; *T_out, *rows_out are then the fastest of the others.  Allocates a copy of the state;
- * synchronous.  The paper's grids (Sec. 6.2: 500^2 to 2000^2) are small
- * enough to stay in L2, where the best tiling differs from the 4096^2
- * default. */
+ * of these (*T_out: its steps between exchanges, *rows_out:
+ * GBSW_SW_ONE_LAUNCH).  Allocates a copy of the state; synchronous.  The
+ * paper's grids (Sec. 6.2: 500^2 to 2000^2) are small enough to stay in L2
+ * or on the chip, where the best tiling differs from the 4096^2 default. */
 gbsw_status sw_autotune(gbsw_sw *sw, int trial_steps, int *T_out, int *rows_out);
+
+/* The one-launch path that sw_step takes with the present tiling: plan[0] x
+ * plan[1] tiles, plan[2] steps between exchanges, plan[3] cells per thread;
+ * four zeros if the steps run as launches. */
+gbsw_status sw_get_chip_plan(gbsw_sw *sw, int plan[4]);
 
 /* Release the context and its device memory.  NULL is ignored. */
 void sw_destroy(gbsw_sw *sw);

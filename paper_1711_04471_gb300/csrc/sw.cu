@@ -581,8 +581,18 @@ gbsw_status sw_set_tiling(gbsw_sw *s, int steps_per_launch, int rows)
     if (!s || steps_per_launch < 0 || steps_per_launch > SW_MAX_BLOCKING) return GBSW_ERR_ARG;
     if (rows < 0 && (steps_per_launch < 1 || steps_per_launch > SWT_MAX_T || rows < -swt_max_rows(steps_per_launch)))
         return GBSW_ERR_ARG;
-    s->blocking = steps_per_launch;
-    s->rows = rows;
+    const bool one_launch = rows == GBSW_SW_ONE_LAUNCH && s->chip.cx;
+    s->blocking = one_launch ? 0 : steps_per_launch;
+    s->rows = one_launch ? 0 : rows;
+    return GBSW_OK;
+}
+
+gbsw_status sw_get_chip_plan(gbsw_sw *s, int plan[4])
+{
+    if (!s || !plan) return GBSW_ERR_ARG;
+    const SWChipPlan c = s->blocking == 0 && s->rows == 0 ? s->chip : SWChipPlan{};
+    const int v[4] = {c.cx, c.cy, c.T, c.per};
+    for (int k = 0; k < 4; ++k) plan[k] = c.cx ? v[k] : 0;
     return GBSW_OK;
 }
 
@@ -696,8 +706,8 @@ gbsw_status sw_autotune(gbsw_sw *s, int trial_steps, int *T_out, int *rows_out)
     if (st != GBSW_OK) return st;
     s->blocking = automatic ? 0 : bestT;
     s->rows = automatic ? 0 : best_rows;
-    if (T_out) *T_out = bestT;
-    if (rows_out) *rows_out = best_rows;
+    if (T_out) *T_out = automatic ? s->chip.T : bestT;
+    if (rows_out) *rows_out = automatic ? GBSW_SW_ONE_LAUNCH : best_rows;
     return GBSW_OK;
 }
 

@@ -12,6 +12,9 @@ import numpy as np
 from . import _native as N
 
 
+ONE_LAUNCH = 1 << 30   # rows of set_tiling: all steps of a call in one launch where the grid fits
+
+
 class SW:
     def __init__(self, params: dict, H: np.ndarray, eta0: np.ndarray, stream=None):
         L = N.lib()
@@ -42,11 +45,19 @@ class SW:
 
     def autotune(self, trial_steps: int = 60):
         """Pick the fused depth and the row-segment height (or tile height,
-        rows < 0) by timing them on this grid (the state is restored);
-        returns (T, rows) in the encoding of set_tiling."""
+        rows < 0, or ONE_LAUNCH) by timing them on this grid (the state is
+        restored); returns (T, rows) in the encoding of set_tiling."""
         T, rows = C.c_int(), C.c_int()
         N.check(N.lib().sw_autotune(self._h, int(trial_steps), C.byref(T), C.byref(rows)), "sw_autotune")
         return T.value, rows.value
+
+    def chip_plan(self):
+        """How step runs all steps of a call in one launch with the present
+        tiling: (tiles in x, in y, steps between exchanges, cells per
+        thread); None if the steps run as launches."""
+        plan = (C.c_int * 4)()
+        N.check(N.lib().sw_get_chip_plan(self._h, plan), "sw_get_chip_plan")
+        return tuple(plan) if plan[0] else None
 
     def volume(self):
         v, w = C.c_double(), C.c_double()
