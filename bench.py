@@ -411,7 +411,8 @@ def run_ensemble(args, rank, world, local):
     cells = int(sum(int(n) * int(n) for n in sizes))
     stream = torch.cuda.current_stream()
     b = SWBatch(members, stream=stream)
-    T, rows = b.autotune(trial_steps=60, cache_path=os.environ.get("GBSW_TUNE_CACHE"))  # ~25 ms per candidate
+    b.autotune(trial_steps=60, cache_path=os.environ.get("GBSW_TUNE_CACHE"))  # ~25 ms per candidate
+    T, rows = b.get_tiling()
     per = STEPS_PER_BENCH_STEP
     for _ in range(args.warmup):
         b.step(per)

@@ -288,13 +288,14 @@ gbsw_status sw_batch_get_state(gbsw_sw_batch *b, int m, float *eta, float *u, fl
 
 /* Tiling: fused steps per level (1..4) and rows per work item (8..65536).
  * Until one is set or tuned, sw_batch_step picks the rows from the instances'
- * sizes; get_tiling then reports 3, 128. */
+ * sizes.  get_tiling reports what the next sw_batch_step uses. */
 gbsw_status sw_batch_set_tiling(gbsw_sw_batch *b, int steps_per_level, int rows_per_item);
 gbsw_status sw_batch_get_tiling(gbsw_sw_batch *b, int *steps_per_level, int *rows_per_item);
 
 /* Time every (steps_per_level, rows_per_item) candidate on this batch
  * (state saved and restored), keep the fastest and return it; the rows
- * picked from the sizes are timed too and kept if they are faster still.  If
+ * picked from the sizes are timed too and kept if they are faster still
+ * (sw_batch_get_tiling then reports them).  If
  * cache_path is not NULL the choice is looked up in / appended to that
  * text file, keyed by device name and instance sizes. */
 gbsw_status sw_batch_autotune(gbsw_sw_batch *b, int trial_steps, const char *cache_path, int *steps_per_level,

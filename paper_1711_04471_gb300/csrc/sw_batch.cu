@@ -183,7 +183,7 @@ struct gbsw_sw_batch {
     int *status;
     double *partials, *area, *vol;
     int cur;
-    int T, rows;         // tiling as set, tuned or reported
+    int T, rows;         // tiling as set or tuned
     bool automatic;      // step with depth BATCH_T and pick_rows() instead
     int auto_rows;       // pick_rows(), 0 until computed
     int grid_cache[8];   // co-resident CTAs per T
@@ -452,8 +452,13 @@ gbsw_status sw_batch_set_tiling(gbsw_sw_batch *b, int steps_per_level, int rows_
 gbsw_status sw_batch_get_tiling(gbsw_sw_batch *b, int *steps_per_level, int *rows_per_item)
 {
     if (!b) return GBSW_ERR_ARG;
-    if (steps_per_level) *steps_per_level = b->T;
-    if (rows_per_item) *rows_per_item = b->rows;
+    int rows = b->rows;
+    if (b->automatic) {
+        const gbsw_status st = pick_rows(b, &rows);
+        if (st != GBSW_OK) return st;
+    }
+    if (steps_per_level) *steps_per_level = step_T(b);
+    if (rows_per_item) *rows_per_item = rows;
     return GBSW_OK;
 }
 

@@ -206,11 +206,14 @@ class SWBatch:
         N.check(N.lib().sw_batch_set_tiling(self._h, int(steps_per_level), int(rows_per_item)), "sw_batch_set_tiling")
 
     def get_tiling(self):
+        """(steps per level, rows per item) that the next step uses."""
         t, r = C.c_int(), C.c_int()
         N.check(N.lib().sw_batch_get_tiling(self._h, C.byref(t), C.byref(r)), "sw_batch_get_tiling")
         return t.value, r.value
 
     def autotune(self, trial_steps: int = 12, cache_path: str | None = None):
+        """Keep the fastest tiling (get_tiling); returns the fastest of the
+        fixed candidates, which the automatic rows may have beaten."""
         t, r = C.c_int(), C.c_int()
         cp = None if cache_path is None else cache_path.encode()
         N.check(N.lib().sw_batch_autotune(self._h, int(trial_steps), cp, C.byref(t), C.byref(r)), "sw_batch_autotune")
