@@ -459,6 +459,13 @@ void les_destroy(gbsw_les *les);
 gbsw_status poisson_solve(int nx, int ny, int nz, double dx, float *p, const float *b, double omega, double tol,
                           int max_iter, int check_every, void *stream, int *iters, double *rel_res);
 
+/* How the solves of an nx x ny x nz grid (poisson_solve, les_step) run on the
+ * current device: as one cooperative launch per solve or per check interval
+ * with plan[0] x plan[1] tiles of whole rows in y and z, plan[2] groups of
+ * four cells per thread and colour (0: rows in shared memory) and the checks
+ * inside the launch if plan[3]; four zeros: as half-sweep launches. */
+gbsw_status poisson_tile_plan(int nx, int ny, int nz, int plan[4]);
+
 /* ------------------------------------------------------------------------
  * Learned warm start for the pressure solve: a 3-D convolutional U-Net
  * (not in the paper; SOR from Sec. 6.3.1 still decides the answer).  The

@@ -69,5 +69,6 @@ def declare(L, sig):
     sig(L, "gbsw_debug_bounds", C.c_int, [C.POINTER(C.c_longlong)])
     sig(L, "gbsw_selftest_bounds", C.c_int, [])
     sig(L, "gbsw_selftest_sor_division", C.c_int, [C.c_int, C.POINTER(C.c_ulonglong)])
+    sig(L, "poisson_tile_plan", C.c_int, [C.c_int, C.c_int, C.c_int, ip])
     sig(L, "poisson_solve", C.c_int, [C.c_int, C.c_int, C.c_int, C.c_double, vp, vp, C.c_double, C.c_double,
                                       C.c_int, C.c_int, vp, ip, dp])

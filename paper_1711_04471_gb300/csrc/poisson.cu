@@ -1064,3 +1064,12 @@ extern "C" gbsw_status poisson_solve(int nx, int ny, int nz, double dx, float *p
     if (fixed) return GBSW_OK;
     return host.done && (host.rho <= tol || host.bb < 1e-60) ? GBSW_OK : GBSW_NOT_CONVERGED;
 }
+
+extern "C" gbsw_status poisson_tile_plan(int nx, int ny, int nz, int plan[4])
+{
+    if (nx < 2 || ny < 2 || nz < 2 || (ny & 1) || nx > 8192 || ny > 8192 || nz > 8192 || !plan) return GBSW_ERR_ARG;
+    const SorTilePlan p = sort_plan(nx, ny, nz);
+    const int v[4] = {p.py, p.pz, p.items, p.psm ? 1 : 0};
+    for (int k = 0; k < 4; ++k) plan[k] = p.py ? v[k] : 0;
+    return GBSW_OK;
+}

@@ -158,6 +158,15 @@ def poisson_solve(p, b, dx: float, omega=1.8, tol=1e-6, max_iter=100000, check_e
     return st, it.value, rr.value
 
 
+def poisson_tile_plan(nx: int, ny: int, nz: int):
+    """How the solves of a grid run on the current device: (tiles in y, in z,
+    groups per thread, 1 if the checks are inside the launch); None if as
+    half-sweep launches."""
+    plan = (C.c_int * 4)()
+    N.check(N.lib().poisson_tile_plan(nx, ny, nz, plan), "poisson_tile_plan")
+    return tuple(plan) if plan[0] else None
+
+
 def warm_start_features(p, b, dx: float, f: int, stream=None):
     """Network input of the warm start from CUDA tensors p (float64) and b
     (float32) of shape (nz, ny, nx).  Returns (x, s): x a CUDA float32

@@ -49,3 +49,21 @@ def test_a_step_that_cannot_be_launched_leaves_the_state(SW64, steps):
         after = g.get_state()
     for f in ("eta", "u", "v", "wet"):
         assert np.array_equal(before[f], after[f]), f
+
+
+# |1 - RN(1/d) d| <= 2^-54 (one correction of the quotient) or more (two), and
+# cell sizes past 2^100 either way (plain division)
+@pytest.mark.parametrize("dx,dy", [(10.0, 12.5), (7.3, 3.7), (1.9999, 9.7), (1.3 * 2.0 ** -101, 1.7 * 2.0 ** -102),
+                                   (1.3 * 2.0 ** 101, 1.7 * 2.0 ** 102), (7.3, 1.7 * 2.0 ** 5)])
+def test_every_form_of_the_division_bitwise(SW64, dx, dy):
+    base = inputs.sw_wetdry(n=90, seed=17)
+    inp = inputs.SWInput(90, 90, dx, dy, 0.02 * min(dx, dy), base.H, base.eta0, hmin=base.hmin)
+    o = oracle.SWState(inp.params(), inp.H, inp.eta0).run(150)
+    with SW64(inp.params(), inp.H, inp.eta0) as g:
+        g.step(150)
+        st = g.get_state()
+    assert np.abs(st["u"]).max() > 0 and np.isfinite(st["eta"]).all()
+    assert np.array_equal(st["eta"], o.eta_i)
+    assert np.array_equal(st["u"], o.u_f)
+    assert np.array_equal(st["v"], o.v_f)
+    assert np.array_equal(st["wet"], o.wet_i)
