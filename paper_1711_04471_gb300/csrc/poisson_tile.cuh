@@ -33,9 +33,9 @@
 // Every wait is bounded by a clock
 // budget; a wait that gives up records DEV_TIMEOUT and the CTA returns.
 //
-// Measured, us per iteration (half-sweep launches before, this kernel):
-// 256x256x128 16.6, 13.1; 300x300x90 18.6, 14.0; 256x128x64 8.9, 5.1;
-// 160x96x64 9.9, 3.2; 72x48x40 5.4, 2.2; 16x16x12 4.7, 0.80 (one CTA).
+// Measured, us per iteration (half-sweep launches, this kernel):
+// 256x256x128 16.9, 13.0; 300x300x90 18.3, 14.2; 256x128x64 8.8, 5.2;
+// 160x96x64 10.0, 3.2; 72x48x40 5.4, 2.2; 16x16x12 4.5, 0.75 (one CTA).
 //
 // Checks.  A register tile whose FP64 pressure and right-hand side fit in
 // shared memory too (psm, about 2 M cells) runs the whole solve in one
@@ -328,7 +328,6 @@ __device__ __forceinline__ SorTileDiag sort_diag(const SorDiag &dg, int nx, int 
 
 #define SORT_OKP(idx) GBSW_INBOUNDS((long long)(idx), (long long)d.plane * (d.nz + 2), &g_sor_bounds)
 #define SORT_OK4(idx) GBSW_INBOUNDS((long long)(idx), (long long)d.cplane * (d.nz + 2) - 3, &g_sor_bounds)
-#define SORT_OK1(idx) GBSW_INBOUNDS((long long)(idx), (long long)d.cplane * (d.nz + 2), &g_sor_bounds)
 
 // Behind e and r: the diagonals by kind of group, then (I = 0) the rim rows.
 __device__ __forceinline__ SorTileDiag *sort_diags(const SorTile &T, bool rsmem)
@@ -1215,6 +1214,5 @@ sor_solve_kernel(const __grid_constant__ SorTileArgs A, const __grid_constant__ 
 }
 #undef SORT_OKP
 #undef SORT_OK4
-#undef SORT_OK1
 
 }  // namespace gbsw

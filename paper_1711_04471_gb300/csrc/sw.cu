@@ -284,7 +284,7 @@ size_t chip_smem(int per) { return ((size_t)SWC_ARRAYS * per * SWC_THREADS + 2 *
 // with one tile), and per step 300 of latency and 650 for each cell of a
 // thread (measured: 500x500 4200 cycles, 700x700 7400).  Several tiles exchange
 // after two steps at the earliest: with an exchange in every step the launches
-// are faster (us per step, chip and launches: 900x900 7.1, 6.4; 1100x1020 11.8, 7.6).
+// are faster (us per step, all wet, chip and launches: 900x900 7.1, 6.4; 1100x1020 11.8, 7.6).
 SWChipPlan chip_plan(int nx, int ny)
 {
     SWChipPlan best{};
@@ -389,8 +389,11 @@ bool capturing(const gbsw_sw *s)
 }
 
 // Default depth of the launches: with few rows per segment the shorter
-// pipeline of T = 2 is better (us per step, T = 2 and 3: 500x500 4.8, 5.7;
-// 1000x1000 7.6, 7.9; 1300x1000 8.7, 8.9; 1237x1501 10.4, 9.6).
+// pipeline of T = 2 is better (us per step, T = 2 and 3, 15 % dry: 500x500 5.8,
+// 7.2; 1000x1000 8.1, 9.0; 1300x1000 9.1, 9.8; 1237x1501 10.8, 10.7; 2000x2000
+// 18.0, 18.7; all wet: 1000x1000 7.6, 7.9; 1300x1000 8.7, 8.9; 1237x1501 10.4,
+// 9.6; 2000x2000 17.4, 17.1).  The line lies where the two cross on all-wet
+// grids; beyond it they differ by 4 % at most on partly dry ones.
 int auto_blocking(const gbsw_sw *s) { return (long long)s->d.nx * s->d.ny < 1400000 ? 2 : 3; }
 
 int tiling_T(const gbsw_sw *s) { return s->blocking > 0 ? s->blocking : auto_blocking(s); }

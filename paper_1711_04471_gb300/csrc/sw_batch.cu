@@ -238,8 +238,8 @@ gbsw_status batch_grid(gbsw_sw_batch *b)
 // level.  The co-resident CTAs take the items in ceil(items / CTAs) rounds,
 // each as long as the item's rows and its pipeline's fill (5T).  With 128
 // rows whatever the sizes, most CTAs of a small ensemble had no item: 12
-// grids of 66 .. 471 cells a side 28.0 us per step, now 7.8; 20 grids of
-// 67 .. 916 29.6, 25.3.
+// grids of 79 .. 497 cells a side 27.5 us per step, now 7.6 (16 rows); 20 grids
+// of 73 .. 855 29.0, 17.0 (64 rows).
 gbsw_status pick_rows(gbsw_sw_batch *b, int *rows)
 {
     if (b->auto_rows == 0) {

@@ -15,18 +15,18 @@
 //
 // Each step is three barrier-separated phases over the region, as in
 // sw_tile_kernel, with fewer operations: a face's flux is formed once, with
-// its velocity; a cell publishes its filtered elevation already multiplied
-// by its wet mask, beside the mask; and the phases are branch-free, so that
-// a thread's cells overlap.  Every rounding is the streaming kernel's, so
+// its velocity; a cell publishes its eta* already multiplied by its wet
+// mask, beside the mask; and the phases are branch-free, so that a thread's
+// cells overlap.  Every rounding is the streaming kernel's, so
 // the states are bitwise the same.  (Four cells of a row per thread with
 // packed FP32 operations was slower: 3.2 us per step at 500x500.)
 //
 // What bounds it: the way of a word from SM to SM (about 1 us per exchange)
 // on small grids, the issue slots and shared-memory wavefronts of the phases
 // on large ones.  us per step, the kernel that the autotuner chose before,
-// this one: 100x100 1.19, 0.65; 500x500 2.55, 2.05; 700x700 5.0, 3.6
-// (untuned, the launches took 10 us and more); today's launches, this one:
-// 800x800 5.9, 4.0; 900x900 6.4, 5.7.
+// this one: 100x100 1.18, 0.65; all wet 500x500 2.54, 2.05; 15 % dry 700x700
+// 4.98, 3.72 (untuned, the launches took 10 us and more); today's launches,
+// this one: 800x800 6.7, 4.2 (all wet 5.9, 4.0); 900x900 7.1, 5.7 (6.4, 5.7).
 #pragma once
 
 #include "sw_kernels.cuh"
@@ -37,7 +37,7 @@ constexpr int SWC_THREADS = 512;
 constexpr int SWC_MAX_T = 4;
 constexpr int SWC_GUARD = 2048;        // most columns of a region
 constexpr int SWC_ARRAYS = 6;          // shared FP32 arrays of a region
-constexpr int SWC_MAX_PER = 14;      // cells of a thread: with 15 and 16 the registers spill and the launches are faster
+constexpr int SWC_MAX_PER = 14;        // cells of a thread (13 and 14 spill a few bytes; with 15 and 16 the launches are faster)
 constexpr long long SWC_WAIT_CYCLES = 4000000000LL;  // budget of a wait: about 2 s
 
 // How a grid is cut: cx x cy tiles of tw x th cells (the last ones smaller),

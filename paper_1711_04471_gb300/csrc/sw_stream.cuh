@@ -30,8 +30,8 @@
 // face's flux is formed once, w eta* travels with w, loads and stores are
 // predicated, a wall is a wet threshold of infinity.  With three barriers
 // per row, branches and the fluxes formed on both sides of every face a step
-// took (T = 3) at 4096x4096 75 us, now 57; 2000x2000 23.5, 17.0; 1237x1501
-// 15.2, 9.5.
+// took (T = 3, 15 % of the cells dry) at 4096x4096 74.6 us, now 61.0; 2000x2000
+// 23.6, 18.7; 1237x1501 15.0, 10.7 (all wet: 17.1 and 9.6 for the last two).
 #pragma once
 
 #include <type_traits>

@@ -20,8 +20,8 @@
 // its latency is one load, 3T short phases and one store, which is what
 // the small grids of the paper (500^2 .. 2000^2, a few MB) need.  The phases
 // are bound by issued instructions: forming each face's flux once, instead of
-// on both sides of it, took the step from 9.63 to 8.75 us at 1100x1020 and
-// from 15.4 to 14.0 us at 1237x1501 (T = 2, balanced heights).
+// on both sides of it, took the step from 9.61 to 8.75 us at 1100x1020 (T = 2,
+// 40-row tiles).
 #pragma once
 
 #include "sw_kernels.cuh"

@@ -66,9 +66,10 @@ struct ConvSmem {
     static constexpr int B_BYTES = COUT * CIN * 2;
     static constexpr int STAGE = ((A_BYTES + B_BYTES + 1023) / 1024) * 1024;
     // Taps in flight.  Four leave room for more tiles per SM, whose epilogues
-    // overlap; with few tiles only the ring hides the loads' latency
-    // (16 -> 16 channels: 8192 tiles 75 us with 4, 111 with 9; 64 -> 32, 8 tiles
-    // 13.9 with 4, 12.7 with 9).
+    // overlap; with few tiles only the ring hides the loads' latency, of which
+    // little is left (16 -> 16 channels: 8192 tiles 75 us with 4, 111 with 9;
+    // 32 -> 64, 8 tiles 13.0 with 4, 12.7 with 6).  64 input channels leave room
+    // for four only.
     static constexpr int STAGES = 4;
     static constexpr int FIT = 72 * 1024 / STAGE;  // what leaves room for a weight-gradient CTA on the SM
     static constexpr int DEEP = FIT > 9 ? 9 : FIT < STAGES ? STAGES : FIT;
