@@ -70,8 +70,8 @@ def test_solves_that_give_up_are_reported(N, monkeypatch, shape, kw):
 def test_a_finished_tile_does_not_hide_anothers_timeout(N, monkeypatch):
     """A right-hand side whose square sum is below 1e-60 is solved by the first
     check, so the last block to come to its barrier finishes while the others
-    give up.  Subnormal values, which take longer, make that the first block,
-    the one that writes the solve's result: the report must not depend on it."""
+    give up.  Should that be the first block, the one that writes the solve's
+    result (its subnormal values take longer), the report must be the same."""
     import torch
     from paper_1711_04471_gb300.les import poisson_solve
     b = torch.zeros((96, 96, 128))
